@@ -66,18 +66,6 @@ __global__ void __launch_bounds__(256) k_batch_plan(const BatchItem<R> *items, B
 }
 
 // ---------------------------------------------------------------- push
-template <typename R>
-__device__ __forceinline__ void flush_acc(const Acc<R> &acc, double *dst) {
-  double v[kAccN];
-  acc.values(v);
-#pragma unroll
-  for (int q = 0; q < kAccN; ++q) {
-    if (!__any_sync(0xffffffffu, v[q] != 0.0)) continue;  // rare events: mostly none
-    const double s = warp_sum(v[q]);
-    if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(dst + q, s);
-  }
-}
-
 // What a warp keeps of its current target: the per-target hot constants
 // and the grid and tally views (the run-wide constants are the kernel's
 // parameter Krun, read from the constant bank like the single-target
@@ -124,7 +112,7 @@ k_batch_push(const Consts Krun, const BatchItem<R> *__restrict__ items, BatchDev
     while (wpref_s[tn + 1] <= w) ++tn;
     if (tn != t) {  // warp-uniform: a new target
       if (t >= 0) {
-        flush_acc(acc, tal_s + t * kAccN);
+        acc.flush_warp(tal_s + t * kAccN);
         acc = Acc<R>();
       }
       t = tn;
@@ -158,7 +146,7 @@ k_batch_push(const Consts Krun, const BatchItem<R> *__restrict__ items, BatchDev
         Krun, it.h, it.grid, tab, it.tv, sc, p, it.off + local, local < it.n, acc,
         tal_s + t * kAccN, stage, SORT ? &so : nullptr, SORT ? &it.sshift : nullptr, nullptr);
   }
-  if (t >= 0) flush_acc(acc, tal_s + t * kAccN);
+  if (t >= 0) acc.flush_warp(tal_s + t * kAccN);
   __syncthreads();
   for (int i = threadIdx.x; i < d.n * kAccN; i += blockDim.x)
     if (tal_s[i] != 0.0) atomicAdd(items[i / kAccN].tv.tal + kAccSlot[i % kAccN], tal_s[i]);

@@ -208,6 +208,43 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// A sum of reals with the accuracy of an FP64 sum of them that keeps off the
+// FP64 unit where it can.  GB300 completes two FP64 operations per clock and
+// SM, so one warp-wide FP64 add holds that unit for 16 clocks: the tree sums
+// at the end of a kernel cost microseconds there.  An FP32 sum is carried as
+// a pair (hi, lo) by Knuth's branch-free two-sum (TAOCP vol. 2, 4.2.2), 48
+// bits wide, on the FP32 units.
+template <typename R>
+struct WideSum;
+template <>
+struct WideSum<float> {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = __fadd_rn(hi, x), t = __fadd_rn(s, -hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -t)), __fadd_rn(x, -t)));
+    hi = s;
+  }
+  __device__ __forceinline__ void over_warp() {  // the total, in every lane
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+      add(h);
+      lo = __fadd_rn(lo, l);
+    }
+  }
+  // (an infinite or NaN sum is hi's; lo is NaN then)
+  __device__ __forceinline__ double value() const {
+    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+  }
+};
+template <>
+struct WideSum<double> {
+  double v = 0.0;
+  __device__ __forceinline__ void add(double x) { v += x; }
+  __device__ __forceinline__ void over_warp() { v = warp_sum(v); }
+  __device__ __forceinline__ double value() const { return v; }
+};
+
 // warp-aggregated atomic increment: lanes with equal keys share one atomic
 __device__ __forceinline__ uint32_t agg_inc(uint32_t *ctr, uint32_t key) {
   const unsigned mask = __activemask();

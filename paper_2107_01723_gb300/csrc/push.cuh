@@ -138,9 +138,10 @@ __device__ constexpr int kAccSlot[kAccN] = {
     T_W_FIELD, T_E_DRAG, T_E_ESC, T_E_REFLUX, T_E_XRAY, T_E_XRAY_ABOVE, T_N_ESC,
     T_N_REFLUX, T_N_REFLUX_ABS, T_N_CUT, T_N_EMIT, T_PSTEPS, T_N_NONFINITE};
 
-// the frequent sums stay in registers; the rare ones (escape, reflux,
-// photons, non-finite electrons) go straight into a shared-memory array of
-// kAccN doubles indexed like kAccSlot, so they hold no registers
+// the frequent sums stay in registers until a warp is done; the rare ones
+// (escape, reflux, photons, non-finite electrons) go straight into a
+// shared-memory array of kAccN doubles indexed like kAccSlot, so they hold no
+// registers
 enum AccIndex { A_W = 0, A_DRAG, A_ESC, A_REF, A_X, A_XA, A_N_ESC, A_N_REF, A_N_REFABS, A_N_CUT,
                 A_N_EMIT, A_N_STEPS, A_N_NF };
 
@@ -148,11 +149,21 @@ template <typename R>
 struct Acc {
   R W = 0, drag = 0;
   int n_cut = 0, n_steps = 0;
-  // in the order of kAccSlot (the rare slots are zero here)
-  __device__ __forceinline__ void values(double (&v)[kAccN]) const {
-#pragma unroll
-    for (int q = 0; q < kAccN; ++q) v[q] = 0.0;
-    v[A_W] = (double)W; v[A_DRAG] = (double)drag; v[A_N_CUT] = n_cut; v[A_N_STEPS] = n_steps;
+  // the warp's totals, added by lane 0 to the shared array `dst` of kAccN doubles
+  __device__ __forceinline__ void flush_warp(double *dst) const {
+    const int cut = __reduce_add_sync(0xffffffffu, n_cut);
+    const int steps = __reduce_add_sync(0xffffffffu, n_steps);
+    WideSum<R> w, d;
+    w.add(W);
+    d.add(drag);
+    w.over_warp();
+    d.over_warp();
+    if ((threadIdx.x & 31) == 0) {
+      if (w.value() != 0.0) atomicAdd(dst + A_W, w.value());
+      if (d.value() != 0.0) atomicAdd(dst + A_DRAG, d.value());
+      if (cut) atomicAdd(dst + A_N_CUT, (double)cut);
+      if (steps) atomicAdd(dst + A_N_STEPS, (double)steps);
+    }
   }
 };
 
