@@ -217,7 +217,6 @@ void hpic::fold(const hpic_target_desc &t, const hpic_run_params &r, const hpic_
   K.F_H = MC2 / (dx * dx * dx);
   K.dx3 = dx * dx * dx;
   K.heat_den = K.n_solids == 1 ? Z * ni * KB : ne_tot * KB;
-  K.Tp_fac = (KB / QE) * std::pow(Z, -4.0 / 3.0);
   // Eqs. (A4)-(A6); a compound's free-electron density sum Z* n_i, e-i
   // collision density sum Z*^2 n_i and total ion density
   K.eta_num = K.n_solids == 1 ? t.lambda2 * ME / (t.Zstar * ni * QE * QE)
@@ -228,8 +227,8 @@ void hpic::fold(const hpic_target_desc &t, const hpic_run_params &r, const hpic_
              std::sqrt(ME / 3.0);
   K.eta_max = t.eta_max_ohm_m;
   K.lambda1 = t.lambda1;
-  K.eta_hot_c = K.eta_num / K.A_hot;
-  K.eta_cold_c = t.lambda1 > 0.0 ? K.eta_num / K.B_cold : 0.0;
+  K.eta_hot_T = K.eta_num / (K.A_hot * KB * std::sqrt(KB));
+  K.eta_cold_T = t.lambda1 > 0.0 ? K.eta_num * std::sqrt(KB) / K.B_cold : 0.0;
   // eta = eta_max exactly while tau <= eta_num/eta_max: tau_hot = A_hot (k T)^1.5
   // grows with T, tau_cold = B_cold/sqrt(k T) falls; the band is narrowed by a
   // relative 1e-6 so that inside it the full formula is capped with room to spare

@@ -299,6 +299,7 @@ void fill_items(hpic_batch *b, std::vector<char> &out) {
     std::memset(&it[t], 0, sizeof(it[t]));
     it[t].K = c->K;
     it[t].h = hpic::make_hot<R>(c->K);
+    it[t].f = hpic::make_field<R>(c->K);
     it[t].g = gview<R>(c);
     it[t].tv = tview(c);
     it[t].cnt = c->cnt;
@@ -400,7 +401,7 @@ int hpic_batch_init(hpic_batch **out, int32_t n_targets, const hpic_target_desc 
     eb += 6 * c->vstride;
     jv += 3 * c->vstride;
     cells += c->K.ncell;
-    npref[t + 1] = npref[t] + c->K.nvec;
+    npref[t + 1] = npref[t] + (c->K.nvec + 31) / 32;
     kpref[t + 1] = kpref[t] + c->K.nkeys + 1;
   }
   slots = round_up(slots, 64);
@@ -410,7 +411,7 @@ int hpic_batch_init(hpic_batch **out, int32_t n_targets, const hpic_target_desc 
   }
   b->slots = slots;
   b->cells = cells;
-  b->nodes_total = npref[n_targets];
+  b->nodes_total = 32 * npref[n_targets];
   b->nkeys_total = kpref[n_targets];
 
   // arena: particles (x2), E and B, J, T, eta, heat, tallies, histograms,

@@ -6,28 +6,67 @@
 
 namespace hpic {
 
-// (i, j, k) of node q; node counts stay below 2^31 (checked at creation), so
-// 32-bit division suffices
-__device__ __forceinline__ void node_of(long long q, int nx, int ny, int &i, int &j, int &k) {
-  const unsigned uq = (unsigned)q, sy = (unsigned)nx + 1u, sz = sy * ((unsigned)ny + 1u);
-  const unsigned kk = uq / sz, r = uq - kk * sz, jj = r / sy;
+// (i, j, k) of node q.  The two divisions by the row and plane lengths go
+// through multiplications by rounded-up reciprocals (Granlund & Montgomery,
+// "Division by invariant integers using multiplication", PLDI 1994): exact for
+// the node counts here, below 2^31 (checked at creation).
+template <typename R>
+__device__ __forceinline__ void node_of(const FieldK<R> &K, long long q, int &i, int &j, int &k) {
+  const unsigned uq = (unsigned)q;
+  const unsigned kk = K.by_sz.quotient(uq), r = uq - kk * (unsigned)K.sz;
+  const unsigned jj = K.by_sy.quotient(r);
   k = (int)kk;
   j = (int)jj;
-  i = (int)(r - jj * sy);
+  i = (int)(r - jj * (unsigned)K.sy);
+}
+
+// ---------------------------------------------------------------- FP64 off the FP64 unit
+// GB300 completes two FP64 operations per clock and SM, conversions from and
+// to FP64 included, so a warp-wide one holds the SM's FP64 unit for 16 clocks
+// where an integer instruction takes a fraction of one.  Conversions of
+// positive numbers well inside FP32's range are therefore done on the bits.
+// in_range: a double in [2^-40, 2^60); zero, negative, infinite and NaN
+// values are not (callers take the plain expressions then).
+__device__ __forceinline__ bool in_range(double x) {
+  return (unsigned)(__double2hiint(x) - 0x3d700000) < 0x06400000u;
+}
+// (float)x of an in_range x: round to nearest, ties to even
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned m = __funnelshift_l(lo, hi, 3) - 0xc0000000u;  // 29 bits cut, exponent rebiased
+  return __uint_as_float(m + (((lo << 3) | (m & 1u)) > 0x80000000u ? 1u : 0u));
+}
+// (double)x of a positive normal x
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+// the smaller of two positive numbers, by their bits
+__device__ __forceinline__ double min_positive(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
+}
+// x^(-3/2) of an in_range x: an FP32 estimate y, then y (1 - e)^(-1/2) with
+// e = 1 - x^3 y^2 (about 1e-6) to second order, the next term being below
+// 1e-18: eight FP64 operations, where rsqrt(x) cubed takes about fourteen
+__device__ __forceinline__ double pow_m32(double x) {
+  const float r = rsqrtf(narrow(x));
+  const double y = widen(r * r * r);
+  const double e = fma(-(x * x * x), y * y, 1.0);
+  return fma(y, e * fma(0.375, e, 0.5), y);
 }
 
 // ---------------------------------------------------------------- E, Eq. (A2)
 // E on the three edges owned by node q (tangential E = 0 on the walls)
 template <typename R>
-__device__ __forceinline__ void efield_node(const Consts &K, const GView<R> &g, long long q) {
+__device__ __forceinline__ void efield_node(const FieldK<R> &K, const GView<R> &g, long long q) {
   const int nx = K.nx, ny = K.ny, nz = K.nz;
-  const int sy = nx + 1;
-  const long long sz = (long long)(nx + 1) * (ny + 1);
+  const int sy = K.sy;
+  const long long sz = K.sz;
   const long long cy = nx, cz = (long long)nx * ny;
-  const R Fc = R(K.F_curl), Fj = R(K.F_j);
+  const R Fc = K.F_curl, Fj = K.F_j;
   const R *Bx = g.B[0], *By = g.B[1], *Bz = g.B[2];
   int i, j, k;
-  node_of(q, nx, ny, i, j, k);
+  node_of(K, q, i, j, k);
   R ex = 0, ey = 0, ez = 0;
   const long long c = i + cy * j + cz * k;  // cell (i, j, k)
   if (i < nx && j >= 1 && j <= ny - 1 && k >= 1 && k <= nz - 1) {
@@ -50,77 +89,71 @@ __device__ __forceinline__ void efield_node(const Consts &K, const GView<R> &g, 
   g.E[2][q] = ez;
 }
 
-// T + rho / (Z n_i k_B C(T)) with the heat capacity of Eq. (A8),
+// rho / (Z n_i k_B C(T)) with the heat capacity of Eq. (A8),
 // C = 0.3 + 1.2 T'(2.2 + T')/(1.1 + T')^2, T' = (k_B T/e) Z^(-4/3), brought
-// over one denominator (one FP64 division per cell)
-__device__ __forceinline__ double heated(const Consts &K, double T, double rho) {
+// over one denominator (one division per cell), in the field precision: in
+// the FP32-mixed path the increment carries a relative error of ~1e-7 of
+// itself; T itself accumulates in FP64
+template <typename R>
+__device__ __forceinline__ R heat_increment(const FieldK<R> &K, R T, R rho) {
   if (K.n_solids == 1) {
-    const double tp = T * K.Tp_fac, D = 1.1 + tp;
-    const double D2 = D * D;
-    return T + rho * D2 / (K.heat_den * (0.3 * D2 + 1.2 * tp * (2.2 + tp)));
+    const R tp = T * K.Tp_fac[0], D = R(1.1) + tp;
+    const R D2 = D * D;
+    return rho * D2 / (K.heat_den * (R(0.3) * D2 + R(1.2) * tp * (R(2.2) + tp)));
   }
   // a compound: heat_den = k_B sum Z n_i, 1/C averaged with the n_e weights
-  double inv_c = 0.0;
+  R inv_c = R(0);
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
     if (s >= K.n_solids) break;
-    const double tp = T * K.Tp_fac_s[s], D = 1.1 + tp;
-    const double D2 = D * D;
-    inv_c += K.ne_frac[s] * D2 / (0.3 * D2 + 1.2 * tp * (2.2 + tp));
+    const R tp = T * K.Tp_fac[s], D = R(1.1) + tp;
+    const R D2 = D * D;
+    inv_c += K.ne_frac[s] * D2 / (R(0.3) * D2 + R(1.2) * tp * (R(2.2) + tp));
   }
-  return T + rho * inv_c / K.heat_den;
-}
-
-// The FP32-mixed path: the increment rho / (n k_B C(T)) of the same
-// expression in FP32 (relative error ~1e-7 of the increment); T itself
-// accumulates in FP64
-__device__ __forceinline__ float heat_increment_f32(const Consts &K, double T, float rho) {
-  const float Tf = (float)T;
-  if (K.n_solids == 1) {
-    const float tp = Tf * (float)K.Tp_fac, D = 1.1f + tp;
-    const float D2 = D * D;
-    return rho * D2 / ((float)K.heat_den * (0.3f * D2 + 1.2f * tp * (2.2f + tp)));
-  }
-  float inv_c = 0.0f;
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    if (s >= K.n_solids) break;
-    const float tp = Tf * (float)K.Tp_fac_s[s], D = 1.1f + tp;
-    const float D2 = D * D;
-    inv_c += (float)K.ne_frac[s] * D2 / (0.3f * D2 + 1.2f * tp * (2.2f + tp));
-  }
-  return rho * inv_c / (float)K.heat_den;
+  return rho * inv_c / K.heat_den;
 }
 
 // reduced Lee-More resistivity, Eqs. (A4)-(A6), capped; inside the band
 // where the cap holds, the cap itself.  eta_num / max(tau_hot, tau_cold) is
-// the smaller of eta_num/(A_hot (kT)^1.5) and eta_num sqrt(kT)/B_cold, both
-// formed from one reciprocal square root (no FP64 division)
-__device__ __forceinline__ double resistivity(const Consts &K, double T) {
-  if (T > K.eta_Tlo && T < K.eta_Thi) return K.eta_max;
-  const double kT = 1.380649e-23 * T;
-  const double r = rsqrt(kT);
-  double eta = K.eta_hot_c * (r * r * r);
-  if (K.lambda1 > 0.0) {
-    const double ec = K.eta_cold_c * (kT * r);
+// the smaller of eta_num/(A_hot (kT)^1.5) and eta_num sqrt(kT)/B_cold.
+// In range, both come from p = T^(-3/2) (sqrt(T) = T^2 p) without a division,
+// a root or a compare on the FP64 unit (Tf = (float)T tells the band, whose
+// float ends lie inside the exact one, where the formula gives the cap too):
+// this and the conversions took the heating of 128^3 cells from 128 to 71 us,
+// and of a 16-target batch of 7.9e6 cells (each with its constants in shared
+// memory and its Ohmic sums made in the warp) from 542 to 199 us.
+__device__ __forceinline__ double resistivity(const FieldCommon &K, double T, float Tf) {
+  if (Tf > K.eta_Tlo && Tf < K.eta_Thi) return K.eta_max;
+  const double p = pow_m32(T);
+  double eta = K.eta_hot * p;
+  if (K.eta_cold > 0.0) eta = min_positive(eta, K.eta_cold * (T * T * p));
+  return min_positive(eta, K.eta_max);
+}
+// the same for any T
+__device__ __noinline__ double resistivity_any(double eta_hot, double eta_cold, double eta_max,
+                                               double T) {
+  const double r = rsqrt(T);
+  double eta = eta_hot * (r * r * r);
+  if (eta_cold > 0.0) {
+    const double ec = eta_cold * (T * r);
     eta = ec < eta ? ec : eta;
   }
-  return eta < K.eta_max ? eta : K.eta_max;
+  return eta < eta_max ? eta : eta_max;
 }
 
 // ---------------------------------------------------------------- B, Eq. (A3), and heating
-// Faraday on the faces owned by node q, then heating of cell q; returns the
-// cell's Ohmic energy (J)
+// Faraday on the faces owned by node q, then heating of cell q; the cell's
+// Ohmic energy density (J/m^3) goes to `ohm`
 template <typename R>
-__device__ __forceinline__ double bheat_node(const Consts &K, const GView<R> &g, long long q) {
+__device__ __forceinline__ void bheat_node(const FieldK<R> &K, const GView<R> &g, long long q,
+                                           WideSum<R> &ohm) {
   const int nx = K.nx, ny = K.ny, nz = K.nz;
-  const int sy = nx + 1;
-  const long long sz = (long long)(nx + 1) * (ny + 1);
-  const R cdt = R(K.cdt_dx);
+  const int sy = K.sy;
+  const long long sz = K.sz;
+  const R cdt = K.cdt;
   const R *Ex = g.E[0], *Ey = g.E[1], *Ez = g.E[2];
-  double e_ohm = 0.0;
   int i, j, k;
-  node_of(q, nx, ny, i, j, k);
+  node_of(K, q, i, j, k);
   if (K.physics & P_FARADAY) {
     if (j < ny && k < nz) g.B[0][q] -= cdt * ((Ez[q + sy] - Ez[q]) - (Ey[q + sz] - Ey[q]));
     if (i < nx && k < nz) g.B[1][q] -= cdt * ((Ex[q + sz] - Ex[q]) - (Ez[q + 1] - Ez[q]));
@@ -140,26 +173,27 @@ __device__ __forceinline__ double bheat_node(const Consts &K, const GView<R> &g,
     }
     // a cell without drag heat or current keeps T and eta (and adds no
     // Ohmic energy) unless e-i equilibration moves it
-    if (Hc == 0.0 && jb2 == R(0) && !(K.physics & P_EI)) return e_ohm;
+    const bool no_heat = (__double_as_longlong(Hc) << 1) == 0;  // +0 or -0
+    if (no_heat && jb2 == R(0) && !(K.physics & P_EI)) return;
     double Te = g.T[c];
     bool changed = false;
-    if constexpr (sizeof(R) == 4) {
-      const float ro = g.eta_r[c] * (float)K.F_ohm * jb2;
-      const float rho = (float)(Hc * K.F_H) + ro;
-      e_ohm = (double)ro * K.dx3;
-      if ((K.physics & P_HEATING) && rho != 0.0f) {  // rho = 0 leaves T as it is
-        Te += (double)heat_increment_f32(K, Te, rho);
-        changed = true;
+    const R ro = g.eta_r[c] * K.F_ohm * jb2;
+    ohm.add(ro);
+    R rho = ro;
+    if (!no_heat) {
+      const double h = Hc * K.F_H;
+      if constexpr (sizeof(R) == 4) rho += in_range(h) ? narrow(h) : (float)h;
+      else rho += h;
+    }
+    if ((K.physics & P_HEATING) && rho != R(0)) {  // rho = 0 leaves T as it is
+      if constexpr (sizeof(R) == 4) {
+        const float Tf = in_range(Te) ? narrow(Te) : (float)Te;
+        const float d = heat_increment<R>(K, Tf, rho);
+        Te += d > 1e-30f && d < 1e30f ? widen(d) : (double)d;
+      } else {
+        Te += heat_increment<R>(K, Te, rho);
       }
-    } else {
-      double rho = Hc * K.F_H;
-      const double ro = g.eta[c] * K.F_ohm * (double)jb2;
-      e_ohm = ro * K.dx3;
-      rho += ro;
-      if ((K.physics & P_HEATING) && rho != 0.0) {  // rho = 0 leaves T as it is
-        Te = heated(K, Te, rho);
-        changed = true;
-      }
+      changed = true;
     }
     // e-i equilibration over the step (App. A): with a = rate_e dt and
     // b = rate_i dt frozen, the gap d = T_e - T_i decays by exp(-(a + b)) and
@@ -178,13 +212,17 @@ __device__ __forceinline__ double bheat_node(const Consts &K, const GView<R> &g,
       }
     }
     if (changed) {  // eta(T) follows T_e
-      const double e = resistivity(K, Te);
+      double e;
+      if (in_range(Te)) {
+        e = resistivity(K, Te, narrow(Te));
+      } else {
+        e = resistivity_any(K.eta_hot, K.eta_cold, K.eta_max, Te);
+      }
       g.T[c] = Te;
       g.eta[c] = e;
-      if constexpr (sizeof(R) == 4) g.eta_r[c] = R(e);
+      if constexpr (sizeof(R) == 4) g.eta_r[c] = in_range(e) ? narrow(e) : (float)e;
     }
   }
-  return e_ohm;
 }
 
 }  // namespace hpic

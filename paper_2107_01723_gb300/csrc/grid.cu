@@ -13,70 +13,102 @@
 namespace hpic {
 
 template <typename R>
-__global__ void __launch_bounds__(256, kFieldBlocksPerSm) k_efield(const Consts K, GView<R> g) {
+__global__ void __launch_bounds__(256, kFieldBlocksPerSm) k_efield(const FieldK<R> K, GView<R> g) {
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < K.nvec;
        q += (long long)gridDim.x * blockDim.x)
     efield_node(K, g, q);
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256, kFieldBlocksPerSm) k_bheat(const Consts K, GView<R> g, TallyView tv) {
-  __shared__ double smem[32];
-  double e_ohm = 0.0;
+__global__ void __launch_bounds__(256, kFieldBlocksPerSm)
+k_bheat(const FieldK<R> K, GView<R> g, TallyView tv) {
+  __shared__ double sum;
+  if (threadIdx.x == 0) sum = 0.0;
+  __syncthreads();
+  WideSum<R> ohm;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < K.nvec;
        q += (long long)gridDim.x * blockDim.x)
-    e_ohm += bheat_node(K, g, q);
-  const double v[1] = {e_ohm};
-  const int slot[1] = {T_E_OHMIC};
-  block_flush<1>(v, slot, tv.tal, smem);
+    bheat_node(K, g, q, ohm);
+  ohm.over_warp();
+  if ((threadIdx.x & 31) == 0 && ohm.value() != 0.0) atomicAdd(&sum, ohm.value());
+  __syncthreads();
+  if (threadIdx.x == 0 && sum != 0.0) atomicAdd(tv.tal + T_E_OHMIC, sum * K.dx3);
 }
 
 // ---------------------------------------------------------------- batched field kernels
-// The targets' node ranges are concatenated (prefix d.npref); a thread walks
-// its grid-stride nodes in increasing order, so its target index only moves
-// forward.  Shared memory holds the prefix and the per-target Ohmic sums.
-__device__ __forceinline__ int advance_target(const long long *pref, int t, int n, long long q) {
-  while (t + 1 < n && pref[t + 1] <= q) ++t;
-  return t;
+// The targets' nodes go in pieces of 32, a warp to a piece (prefix d.npref),
+// so a warp's nodes are of one target; a warp walks its pieces in increasing
+// order and keeps its target's constants and views in shared memory.
+template <typename R>
+struct FieldHot {
+  FieldK<R> K;
+  GView<R> g;
+};
+
+template <typename R>
+__device__ __forceinline__ int enter_target(FieldHot<R> &w, const BatchItem<R> *items,
+                                            const long long *pref, int t, long long piece) {
+  int tn = t < 0 ? 0 : t;
+  while (pref[tn + 1] <= piece) ++tn;
+  if (tn != t) {  // warp-uniform
+    static_assert(sizeof(FieldK<R>) % 4 == 0 && sizeof(GView<R>) % 4 == 0, "copied by words");
+    __syncwarp();
+    auto copy = [&](void *dst, const void *from, int bytes) {
+      const uint32_t *a = static_cast<const uint32_t *>(from);
+      uint32_t *b = static_cast<uint32_t *>(dst);
+      for (int k = threadIdx.x & 31; k < bytes / 4; k += 32) b[k] = __ldg(a + k);
+    };
+    copy(&w.K, &items[tn].f, (int)sizeof(FieldK<R>));
+    copy(&w.g, &items[tn].g, (int)sizeof(GView<R>));
+    __syncwarp();
+  }
+  return tn;
 }
 
 template <typename R>
 __global__ void __launch_bounds__(256, kBatchFieldBlocksPerSm)
 k_batch_efield(const BatchItem<R> *items, BatchDev d) {
   extern __shared__ long long npref_s[];
+  __shared__ FieldHot<R> hot[8];
   for (int t = threadIdx.x; t <= d.n; t += blockDim.x) npref_s[t] = d.npref[t];
   __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long N = npref_s[d.n];
-  int t = 0;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < N;
-       q += (long long)gridDim.x * blockDim.x) {
-    t = advance_target(npref_s, t, d.n, q);
-    efield_node(items[t].K, items[t].g, q - npref_s[t]);
+  int t = -1;
+  for (long long w = blockIdx.x * 8ll + warp; w < N; w += gridDim.x * 8ll) {
+    t = enter_target(hot[warp], items, npref_s, t, w);
+    const long long q = (w - npref_s[t]) * 32 + lane;
+    if (q < hot[warp].K.nvec) efield_node(hot[warp].K, hot[warp].g, q);
   }
 }
 
+// (Each thread used to add its FP64 Ohmic sum to its target's shared double,
+// a compare-and-swap loop of up to 256 threads on one address.)
 template <typename R>
 __global__ void __launch_bounds__(256, kBatchFieldBlocksPerSm)
 k_batch_bheat(const BatchItem<R> *items, BatchDev d) {
   extern __shared__ long long npref_s[];
+  __shared__ FieldHot<R> hot[8];
   double *ohm_s = reinterpret_cast<double *>(npref_s + d.n + 1);
   for (int t = threadIdx.x; t <= d.n; t += blockDim.x) npref_s[t] = d.npref[t];
   for (int t = threadIdx.x; t < d.n; t += blockDim.x) ohm_s[t] = 0.0;
   __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long N = npref_s[d.n];
-  int t = 0;
-  double e_ohm = 0.0;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < N;
-       q += (long long)gridDim.x * blockDim.x) {
-    const int tn = advance_target(npref_s, t, d.n, q);
-    if (tn != t) {
-      if (e_ohm != 0.0) atomicAdd(ohm_s + t, e_ohm);
-      e_ohm = 0.0;
-      t = tn;
-    }
-    e_ohm += bheat_node(items[t].K, items[t].g, q - npref_s[t]);
+  int t = -1;
+  WideSum<R> ohm;
+  auto flush = [&]() {  // the warp's sum to its target's
+    ohm.over_warp();
+    if (lane == 0 && ohm.value() != 0.0) atomicAdd(ohm_s + t, ohm.value() * hot[warp].K.dx3);
+    ohm = WideSum<R>();
+  };
+  for (long long w = blockIdx.x * 8ll + warp; w < N; w += gridDim.x * 8ll) {
+    if (t >= 0 && npref_s[t + 1] <= w) flush();
+    t = enter_target(hot[warp], items, npref_s, t, w);
+    const long long q = (w - npref_s[t]) * 32 + lane;
+    if (q < hot[warp].K.nvec) bheat_node(hot[warp].K, hot[warp].g, q, ohm);
   }
-  if (e_ohm != 0.0) atomicAdd(ohm_s + t, e_ohm);
+  if (t >= 0) flush();
   __syncthreads();
   for (int u = threadIdx.x; u < d.n; u += blockDim.x)
     if (ohm_s[u] != 0.0) atomicAdd(items[u].tv.tal + T_E_OHMIC, ohm_s[u]);
@@ -319,12 +351,12 @@ __global__ void __launch_bounds__(256) k_field_energy(const Consts K, GView<R> g
 // ---------------------------------------------------------------- launchers
 template <typename R>
 void launch_efield(const Consts &K, GView<R> g, int grid, cudaStream_t st) {
-  k_efield<R><<<grid, 256, 0, st>>>(K, g);
+  k_efield<R><<<grid, 256, 0, st>>>(make_field<R>(K), g);
 }
 
 template <typename R>
 void launch_bheat(const Consts &K, GView<R> g, TallyView tv, int grid, cudaStream_t st) {
-  k_bheat<R><<<grid, 256, 0, st>>>(K, g, tv);
+  k_bheat<R><<<grid, 256, 0, st>>>(make_field<R>(K), g, tv);
 }
 
 int launch_scan(uint32_t *counts, long long m, uint32_t *partials, cudaStream_t st) {

@@ -84,6 +84,75 @@ inline HotK<R> make_hot(const Consts &K) {
   return h;
 }
 
+// n / d of n < 2^31 as a multiplication (see node_of)
+struct Quotient {
+  uint32_t m;  // floor(2^(31 + s) / d) + 1, s = ceil(log2 d)
+  int sh;      // s - 1
+  __device__ __forceinline__ unsigned quotient(unsigned n) const { return __umulhi(n, m) >> sh; }
+};
+inline Quotient make_quotient(uint32_t d) {  // d >= 2
+  int s = 1;
+  while ((1ull << s) < d) ++s;
+  return Quotient{(uint32_t)((1ull << (31 + s)) / d + 1), s - 1};
+}
+
+// what the field and heating kernels need of one target: the sizes, and the
+// constants in the precision each is used in, so that no conversion runs per
+// node (an FP64 conversion costs as much as an FP64 operation there)
+struct FieldCommon {
+  int nx, ny, nz, sy, sz;  // sy, sz: nodes per row and plane
+  int physics, n_solids;
+  Quotient by_sy, by_sz;
+  long long nvec;
+  double F_H, dx3;
+  double eta_hot, eta_cold, eta_max;  // eta = min(eta_hot T^-1.5, eta_cold T^0.5, eta_max), T in K
+  float eta_Tlo, eta_Thi;             // eta(T) is at its cap in this band
+  double ei_a, ei_mi, ei_me, Zstar, fs_q, fs_c;
+};
+template <typename R>
+struct FieldK : FieldCommon {
+  R F_curl, F_j, cdt, F_ohm, heat_den;
+  R Tp_fac[4], ne_frac[4];  // per element
+};
+template <typename R>
+inline FieldK<R> make_field(const Consts &K) {
+  FieldK<R> f{};
+  f.nx = K.nx;
+  f.ny = K.ny;
+  f.nz = K.nz;
+  f.sy = K.nx + 1;
+  f.sz = (K.nx + 1) * (K.ny + 1);
+  f.physics = K.physics;
+  f.n_solids = K.n_solids;
+  f.by_sy = make_quotient((uint32_t)f.sy);
+  f.by_sz = make_quotient((uint32_t)f.sz);
+  f.nvec = K.nvec;
+  f.F_H = K.F_H;
+  f.dx3 = K.dx3;
+  f.eta_hot = K.eta_hot_T;
+  f.eta_cold = K.eta_cold_T;
+  f.eta_max = K.eta_max;
+  // the exact band's ends moved inwards by more than a float's rounding
+  f.eta_Tlo = (float)(K.eta_Tlo * (1.0 + 5e-7));
+  f.eta_Thi = (float)(K.eta_Thi * (1.0 - 5e-7));
+  f.ei_a = K.ei_a;
+  f.ei_mi = K.ei_mi;
+  f.ei_me = K.ei_me;
+  f.Zstar = K.Zstar;
+  f.fs_q = K.fs_q;
+  f.fs_c = K.fs_c;
+  f.F_curl = R(K.F_curl);
+  f.F_j = R(K.F_j);
+  f.cdt = R(K.cdt_dx);
+  f.F_ohm = R(K.F_ohm);
+  f.heat_den = R(K.heat_den);
+  for (int s = 0; s < 4; ++s) {
+    f.Tp_fac[s] = R(K.Tp_fac_s[s]);
+    f.ne_frac[s] = R(K.ne_frac[s]);
+  }
+  return f;
+}
+
 // message returned by hpic_last_error(NULL) (entry points without a context)
 void set_global_error(const char *msg);
 
@@ -219,6 +288,7 @@ template <typename R>
 struct BatchItem {
   Consts K;
   HotK<R> h;
+  FieldK<R> f;
   GView<R> g;
   TallyView tv;
   Counters *cnt;
@@ -230,7 +300,7 @@ struct BatchDev {
   int n;                  // targets
   long long *wpref;       // warp-sized particle tasks, from the live counts
   long long *ipref;       // electrons injected in this step
-  const long long *npref; // vector-grid nodes
+  const long long *npref; // warp-sized (32-node) pieces of the vector grids
   const long long *kpref; // sort keys (each target's tile keys, then its dead bin)
   long long *sstart;      // sort: first sorted offset of each target (n entries)
   long long *snew;        // sort: slots kept per target (n entries)
