@@ -168,6 +168,31 @@ __device__ __forceinline__ double m_fcos2pi(double u) { return cospi(2.0 * u); }
 __device__ __forceinline__ float m_floor(float x) { return floorf(x); }
 __device__ __forceinline__ double m_floor(double x) { return floor(x); }
 
+// ---------------------------------------------------------------- FP64 off the FP64 unit
+// GB300 completes two FP64 operations per clock and SM, conversions from and
+// to FP64 included, so a warp-wide one holds the SM's FP64 unit for 16 clocks
+// where an integer instruction takes a fraction of one.  Conversions of
+// positive numbers well inside FP32's range are therefore done on the bits.
+// in_range: a double in [2^-40, 2^60); zero, negative, infinite and NaN
+// values are not (callers take the plain expressions then).
+__device__ __forceinline__ bool in_range(double x) {
+  return (unsigned)(__double2hiint(x) - 0x3d700000) < 0x06400000u;
+}
+// (float)x of an in_range x: round to nearest, ties to even
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned m = __funnelshift_l(lo, hi, 3) - 0xc0000000u;  // 29 bits cut, exponent rebiased
+  return __uint_as_float(m + (((lo << 3) | (m & 1u)) > 0x80000000u ? 1u : 0u));
+}
+// (double)x of a positive normal x
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+// the smaller of two positive numbers, by their bits
+__device__ __forceinline__ double min_positive(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
+}
 // Sort key of cell (i, j, k): 4x4x4 tiles in x-fastest tile order, cells
 // x-fastest inside a tile, so consecutive electrons share a compact box.
 __host__ __device__ __forceinline__ uint32_t tile_key(int i, int j, int k, int nti, int ntj) {

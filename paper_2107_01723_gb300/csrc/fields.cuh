@@ -20,31 +20,6 @@ __device__ __forceinline__ void node_of(const FieldK<R> &K, long long q, int &i,
   i = (int)(r - jj * (unsigned)K.sy);
 }
 
-// ---------------------------------------------------------------- FP64 off the FP64 unit
-// GB300 completes two FP64 operations per clock and SM, conversions from and
-// to FP64 included, so a warp-wide one holds the SM's FP64 unit for 16 clocks
-// where an integer instruction takes a fraction of one.  Conversions of
-// positive numbers well inside FP32's range are therefore done on the bits.
-// in_range: a double in [2^-40, 2^60); zero, negative, infinite and NaN
-// values are not (callers take the plain expressions then).
-__device__ __forceinline__ bool in_range(double x) {
-  return (unsigned)(__double2hiint(x) - 0x3d700000) < 0x06400000u;
-}
-// (float)x of an in_range x: round to nearest, ties to even
-__device__ __forceinline__ float narrow(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned m = __funnelshift_l(lo, hi, 3) - 0xc0000000u;  // 29 bits cut, exponent rebiased
-  return __uint_as_float(m + (((lo << 3) | (m & 1u)) > 0x80000000u ? 1u : 0u));
-}
-// (double)x of a positive normal x
-__device__ __forceinline__ double widen(float x) {
-  const unsigned b = __float_as_uint(x);
-  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
-}
-// the smaller of two positive numbers, by their bits
-__device__ __forceinline__ double min_positive(double a, double b) {
-  return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
-}
 // x^(-3/2) of an in_range x: an FP32 estimate y, then y (1 - e)^(-1/2) with
 // e = 1 - x^3 y^2 (about 1e-6) to second order, the next term being below
 // 1e-18: eight FP64 operations, where rsqrt(x) cubed takes about fourteen
@@ -130,7 +105,7 @@ __device__ __forceinline__ double resistivity(const FieldCommon &K, double T, fl
   return min_positive(eta, K.eta_max);
 }
 // the same for any T
-__device__ __noinline__ double resistivity_any(double eta_hot, double eta_cold, double eta_max,
+inline __device__ __noinline__ double resistivity_any(double eta_hot, double eta_cold, double eta_max,
                                                double T) {
   const double r = rsqrt(T);
   double eta = eta_hot * (r * r * r);
