@@ -193,6 +193,70 @@ __device__ __forceinline__ double widen(float x) {
 __device__ __forceinline__ double min_positive(double a, double b) {
   return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
 }
+
+// Reciprocals and roots for the per-electron arithmetic, of normal numbers
+// well inside FP32's range (others take the plain expressions in FP64; in
+// FP32 callers keep to x > 0).
+// FP32: the hardware estimate (m_rcp, m_rsqrt: 1-2 ulp), or one Newton step on
+// its residual formed with a fused multiply-add (m_*_near: the rounded result
+// but for rare last bits, without the range tests of the rounded functions),
+// where no rounding bias may enter an energy that no tally records.
+// FP64: from the FP32 estimate by one step of the series in the residual e
+// (about 1e-7), to e^2: three operations for 1/x, five for x^(-1/2), of a unit
+// that completes two per clock and SM.
+__device__ __forceinline__ bool fp32_range(double x) {  // [2^-100, 2^100)
+  return (unsigned)(__double2hiint(x) - 0x39b00000) < 0x0c800000u;
+}
+__device__ __forceinline__ float m_rcp(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ double m_rcp(double x) {
+  if (!fp32_range(x)) return 1.0 / x;
+  const double y = widen(__fdividef(1.0f, narrow(x)));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float m_rsqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double m_rsqrt(double x) {
+  if (!fp32_range(x)) return rsqrt(x);
+  const double y = widen(rsqrtf(narrow(x)));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y, e * fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ float m_rsqrt_near(float x) {
+  const float r = rsqrtf(x);
+  return fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
+}
+__device__ __forceinline__ double m_rsqrt_near(double x) { return m_rsqrt(x); }
+__device__ __forceinline__ float m_sqrt_near(float x) {
+  const float r = rsqrtf(x), s = x * r;
+  return fmaf(fmaf(-s, s, x), 0.5f * r, s);
+}
+__device__ __forceinline__ double m_sqrt_near(double x) { return x * m_rsqrt(x); }
+__device__ __forceinline__ float m_div_near(float n, float d) {
+  const float y = __fdividef(1.0f, d), q = n * y;
+  return fmaf(fmaf(-q, d, n), y, q);
+}
+__device__ __forceinline__ double m_div_near(double n, double d) { return n * m_rcp(d); }
+// sine and cosine of a deflection: by their series up to |x| = 1 (to x^11 and
+// x^12 in FP32: below 1e-9), where nearly all are
+__device__ __forceinline__ void m_sincos_small(float x, float *s, float *c) {
+  if (fabsf(x) <= 1.0f) {
+    const float t = x * x;
+    float p = fmaf(t, -1.0f / 39916800.0f, 1.0f / 362880.0f);
+    p = fmaf(t, p, -1.0f / 5040.0f);
+    p = fmaf(t, p, 1.0f / 120.0f);
+    p = fmaf(t, p, -1.0f / 6.0f);
+    *s = fmaf(x * t, p, x);
+    float q = fmaf(t, -1.0f / 3628800.0f, 1.0f / 40320.0f);
+    q = fmaf(t, q, -1.0f / 720.0f);
+    q = fmaf(t, q, 1.0f / 24.0f);
+    q = fmaf(t, q, -0.5f);
+    *c = fmaf(t, q, 1.0f);
+  } else {
+    sincosf(x, s, c);
+  }
+}
+__device__ __forceinline__ void m_sincos_small(double x, double *s, double *c) { sincos(x, s, c); }
+
 // Sort key of cell (i, j, k): 4x4x4 tiles in x-fastest tile order, cells
 // x-fastest inside a tile, so consecutive electrons share a compact box.
 __host__ __device__ __forceinline__ uint32_t tile_key(int i, int j, int k, int nti, int ntj) {
@@ -205,6 +269,13 @@ template <typename R>
 __device__ __forceinline__ R kinetic(R ux, R uy, R uz) {
   const R u2 = ux * ux + uy * uy + uz * uz;
   return m_div_rn(u2, R(1) + m_sqrt_rn(R(1) + u2));
+}
+
+// the same of u^2, with gamma: near-rounded
+template <typename R>
+__device__ __forceinline__ R kinetic_near(R u2, R &gam) {
+  gam = m_sqrt_near(R(1) + u2);
+  return m_div_near(u2, R(1) + gam);
 }
 
 // momentum |u| of kinetic energy e (m_e c^2)
@@ -224,6 +295,21 @@ __device__ __forceinline__ void rotate(R &dx, R &dy, R &dz, R ct, R st, R cp, R 
   const R px = e1x * cp + e2x * sp, py = e1y * cp + e2y * sp, pz = e1z * cp + e2z * sp;
   const R ox = dx * ct + px * st, oy = dy * ct + py * st, oz = dz * ct + pz * st;
   dx = ox; dy = oy; dz = oz;
+}
+
+// The same rotation with the sums over the frame's vectors carried out: with
+// (qx, qy) = st (cp, sp), V = sg dx qx + dy qy and T = a V the rotated
+// direction is (dx (ct + T) + qx, dy (ct + T) + sg qy, dz ct - V).
+template <typename R>
+__device__ __forceinline__ void rotate_near(R &dx, R &dy, R &dz, R ct, R st, R cp, R sp) {
+  const bool up = dz >= R(0);
+  const R qx = st * cp, qy = st * sp;
+  const R V = (up ? dx : -dx) * qx + dy * qy;
+  const R T = m_div_near(V, (up ? R(-1) : R(1)) - dz);
+  const R k = ct + T;
+  dx = dx * k + qx;
+  dy = dy * k + (up ? qy : -qy);
+  dz = dz * ct - V;
 }
 
 // ---------------------------------------------------------------- reductions

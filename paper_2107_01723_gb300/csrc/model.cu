@@ -31,10 +31,8 @@ constexpr double kMC2 = kME * kC * kC;
 // in 19 (measured on chains of DFMA, dependent or not).  So operations are
 // what counts here: divisions start from an FP32 reciprocal, the two
 // logarithms of the ionisation bracket are one, table-driven, comparisons run
-// on the bits.  ok: positive, in FP32's range with room for the products.
-__device__ __forceinline__ bool ok(double x) {
-  return (unsigned)(__double2hiint(x) - 0x39b00000) < 0x0c800000u;  // [2^-100, 2^100)
-}
+// on the bits.
+__device__ __forceinline__ bool ok(double x) { return fp32_range(x); }
 // a < b by the bits, for numbers that are not both negative (a NaN counts as
 // beyond every number of its sign)
 __device__ __forceinline__ bool less(double a, double b) {
