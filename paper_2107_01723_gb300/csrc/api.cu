@@ -76,14 +76,6 @@ int grid_blocks(const hpic_ctx *c, long long work) {
   return (int)(g < 1 ? 1 : g);
 }
 
-// one resident wave of the particle kernel, or the blocks its slots fill
-template <typename R>
-int push_blocks(const hpic_ctx *c) {
-  const long long want = (c->cap + hpic::push_threads<R>() - 1) / hpic::push_threads<R>();
-  const long long cap = (long long)c->sm_count * hpic::push_blocks_per_sm<R>();
-  return (int)(want < cap ? want : cap);
-}
-
 size_t particle_bytes(const hpic_ctx *c, long long stride) {
   return (size_t)stride * (8 * c->rsz + sizeof(uint32_t));  // 7 reals, weight, id
 }
@@ -439,7 +431,6 @@ int step_impl(hpic_ctx *ctx, long long nsteps) {
                            : reinterpret_cast<const R *>(ctx->t64);
   const int gp = grid_blocks(ctx, ctx->cap);
   const int gg = field_blocks(ctx, ctx->K.nvec);
-  const int gpush = push_blocks<R>(ctx);
   const bool grid_on = !(ctx->K.physics & hpic::P_UNBOUNDED);
   for (long long s = 0; s < nsteps; ++s) {
     if (grid_on) {
@@ -491,7 +482,7 @@ int step_impl(hpic_ctx *ctx, long long nsteps) {
       CK(cudaEventRecord(ctx->ev[ctx->ev_used], ctx->stream));
     }
     hpic::launch_push<R>(ctx->K, P(ctx->cur), G, tab, ctx->cnt, tv,
-                         gpush, ctx->stream, so, ko);
+                         ctx->cap, ctx->sm_count, ctx->stream, so, ko);
     ctx->launches += 1;
     if (ctx->prof) {
       CK(cudaEventRecord(ctx->ev[ctx->ev_used + 1], ctx->stream));

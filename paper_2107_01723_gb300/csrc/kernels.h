@@ -173,11 +173,19 @@ std::vector<InjCell> injection_cells(const hpic_target_desc &t, const hpic_laser
 // warps take consecutive slots, so their gathers share L1 lines.  (Against
 // it: five blocks of 256 at 48 registers, 84 B of spills, 3.5 % slower; six
 // of 192 at 56 registers 3.2 %; four of 288 1.2 %; two of 576 level.)  FP64:
-// two blocks of 256.
+// two blocks of 256.  In the unbounded medium FP32 runs three blocks of 512.
+enum PushMode {
+  kPushPlain = 0,  // a plain step
+  kPushKeys = 1,   // one that also computes the next sort's keys (KeyOut)
+  kPushSort = 2,   // one that also sorts (SortOut)
+  kPushFree = 3    // a plain step in an unbounded medium: no gather, no deposit (FP32)
+};
 template <typename R>
-constexpr int push_blocks_per_sm() { return sizeof(R) == 4 ? 3 : 2; }
+constexpr int push_blocks_per_sm(int mode) { return sizeof(R) == 4 ? 3 : 2; }
 template <typename R>
-constexpr int push_threads() { return sizeof(R) == 4 ? 384 : 256; }
+constexpr int push_threads(int mode) {
+  return sizeof(R) == 4 ? (mode == kPushFree ? 512 : 384) : 256;
+}
 // resident 256-thread blocks per SM of the field and heating kernels (their
 // launch bounds); they are launched as one wave of sm_count times this many
 // blocks (grid-stride over the nodes), so no partial second wave trails
@@ -227,14 +235,10 @@ struct KeyOut {
   R lead;
 };
 
-// the push kernel's modes: a plain step, a step that also computes the next
-// sort's keys (KeyOut), a step that also sorts (SortOut)
-enum PushMode { kPushPlain = 0, kPushKeys = 1, kPushSort = 2 };
-
 template <typename R>
 void launch_push(const Consts &K, PView<R> p, GView<R> g, const R *table, Counters *cnt,
-                 TallyView tv, int grid, cudaStream_t st, const SortOut<R> &so,
-                 const KeyOut<R> &ko);
+                 TallyView tv, long long cap, int sm_count, cudaStream_t st,
+                 const SortOut<R> &so, const KeyOut<R> &ko);
 template <typename R>
 void launch_inject(const Consts &K, PView<R> p, Counters *cnt, long long cap, TallyView tv,
                    int grid, cudaStream_t st);

@@ -26,14 +26,14 @@
 
 namespace hpic {
 
-// MODE: a plain step, one that also keys the next sort (ko), or one that
-// also sorts (so says where the electrons go); the other modes' code is
-// compiled out.
+// MODE: a plain step, one that also keys the next sort (ko), one that also
+// sorts (so says where the electrons go), or a plain one in an unbounded
+// medium; the other modes' code is compiled out.
 template <typename R, int NS, int MODE>
 // Launched as one persistent wave in the shape push_threads/push_blocks_per_sm
 // give: the kernel is issue- and latency-bound and gains from the warps, up
 // to the register count at which spills begin.
-__global__ void __launch_bounds__(push_threads<R>(), push_blocks_per_sm<R>())
+__global__ void __launch_bounds__(push_threads<R>(MODE), push_blocks_per_sm<R>(MODE))
 k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__restrict__ tab,
        Counters *cnt, TallyView tv, const SortOut<R> so, const KeyOut<R> ko) {
   const long long n = cnt->n;
@@ -42,7 +42,7 @@ k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__rest
   if (threadIdx.x < kAccN) sums[threadIdx.x] = 0.0;
   __syncthreads();
   extern __shared__ __align__(16) unsigned char dyn[];  // the warps' deposit stages
-  R *stage = reinterpret_cast<R *>(dyn) + (threadIdx.x >> 5) * dep_words<R>();
+  R *stage = reinterpret_cast<R *>(dyn) + (threadIdx.x >> 5) * push_warp_words<R, MODE>();
   StepCtx sc;
   sc.step_ll = cnt->step;
   sc.step = (uint32_t)sc.step_ll;
@@ -57,10 +57,13 @@ k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__rest
   // warp-uniform loop: every lane reaches the warp-cooperative deposits
   const int lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x - lane); base < n;
-       base += stride)
+  const long long first = blockIdx.x * (long long)blockDim.x + (threadIdx.x - lane);
+  if constexpr (reads_ahead<R, MODE>()) {
+    if (first < n) read_ahead(p, first, stage);
+  }
+  for (long long base = first; base < n; base += stride)
     push_warp<R, NS, MODE>(K, h, g, tab, tv, sc, p, base + lane, base + lane < n, acc, sums,
-                           stage, MODE == kPushSort ? &so : nullptr,
+                           stage, base + stride < n ? base + stride : -1, MODE == kPushSort ? &so : nullptr,
                            MODE == kPushSort ? &no_shift : nullptr,
                            MODE == kPushKeys ? &ko : nullptr);
 
@@ -222,8 +225,10 @@ __global__ void k_advance(Counters *cnt, long long cap) {
 
 // ---------------------------------------------------------------- launchers
 
-template <typename R>
-constexpr size_t push_stage_bytes() { return (push_threads<R>() / 32) * dep_words<R>() * sizeof(R); }
+template <typename R, int MODE>
+constexpr size_t push_stage_bytes() {
+  return (push_threads<R>(MODE) / 32) * push_warp_words<R, MODE>() * sizeof(R);
+}
 
 cudaError_t prepare_push() {
   cudaError_t e = cudaSuccess;
@@ -231,43 +236,60 @@ cudaError_t prepare_push() {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  set((const void *)k_push<float, 1, kPushPlain>, push_stage_bytes<float>());
-  set((const void *)k_push<float, 1, kPushKeys>, push_stage_bytes<float>());
-  set((const void *)k_push<float, 1, kPushSort>, push_stage_bytes<float>());
-  set((const void *)k_push<float, 4, kPushPlain>, push_stage_bytes<float>());
-  set((const void *)k_push<float, 4, kPushKeys>, push_stage_bytes<float>());
-  set((const void *)k_push<float, 4, kPushSort>, push_stage_bytes<float>());
-  set((const void *)k_push<double, 1, kPushPlain>, push_stage_bytes<double>());
-  set((const void *)k_push<double, 1, kPushKeys>, push_stage_bytes<double>());
-  set((const void *)k_push<double, 1, kPushSort>, push_stage_bytes<double>());
-  set((const void *)k_push<double, 4, kPushPlain>, push_stage_bytes<double>());
-  set((const void *)k_push<double, 4, kPushKeys>, push_stage_bytes<double>());
-  set((const void *)k_push<double, 4, kPushSort>, push_stage_bytes<double>());
+  set((const void *)k_push<float, 1, kPushPlain>, push_stage_bytes<float, kPushPlain>());
+  set((const void *)k_push<float, 1, kPushKeys>, push_stage_bytes<float, kPushKeys>());
+  set((const void *)k_push<float, 1, kPushSort>, push_stage_bytes<float, kPushSort>());
+  set((const void *)k_push<float, 4, kPushPlain>, push_stage_bytes<float, kPushPlain>());
+  set((const void *)k_push<float, 4, kPushKeys>, push_stage_bytes<float, kPushKeys>());
+  set((const void *)k_push<float, 4, kPushSort>, push_stage_bytes<float, kPushSort>());
+  set((const void *)k_push<double, 1, kPushPlain>, push_stage_bytes<double, kPushPlain>());
+  set((const void *)k_push<double, 1, kPushKeys>, push_stage_bytes<double, kPushKeys>());
+  set((const void *)k_push<double, 1, kPushSort>, push_stage_bytes<double, kPushSort>());
+  set((const void *)k_push<double, 4, kPushPlain>, push_stage_bytes<double, kPushPlain>());
+  set((const void *)k_push<double, 4, kPushKeys>, push_stage_bytes<double, kPushKeys>());
+  set((const void *)k_push<double, 4, kPushSort>, push_stage_bytes<double, kPushSort>());
   return e;
+}
+
+template <typename R, int NS, int MODE>
+void launch_push_mode(const Consts &K, const HotK<R> &h, PView<R> p, GView<R> g, const R *table,
+                      Counters *cnt, TallyView tv, long long cap, int sm_count, cudaStream_t st,
+                      const SortOut<R> &so, const KeyOut<R> &ko) {
+  // one resident wave, or the blocks the slots fill
+  constexpr int threads = push_threads<R>(MODE);
+  const long long want = (cap + threads - 1) / threads;
+  const long long wave = (long long)sm_count * push_blocks_per_sm<R>(MODE);
+  k_push<R, NS, MODE><<<(int)(want < wave ? want : wave), threads, push_stage_bytes<R, MODE>(), st>>>(
+      K, h, p, g, table, cnt, tv, so, ko);
 }
 
 template <typename R, int NS>
 void launch_push_ns(const Consts &K, const HotK<R> &h, PView<R> p, GView<R> g, const R *table,
-                    Counters *cnt, TallyView tv, int grid, cudaStream_t st, const SortOut<R> &so,
-                    const KeyOut<R> &ko) {
-  const size_t sm = push_stage_bytes<R>();
+                    Counters *cnt, TallyView tv, long long cap, int sm_count, cudaStream_t st,
+                    const SortOut<R> &so, const KeyOut<R> &ko) {
+  if constexpr (sizeof(R) == 4) {
+    if ((K.physics & P_UNBOUNDED) && !so.dst.x && !ko.keys) {
+      launch_push_mode<R, NS, kPushFree>(K, h, p, g, table, cnt, tv, cap, sm_count, st, so, ko);
+      return;
+    }
+  }
   if (so.dst.x)
-    k_push<R, NS, kPushSort><<<grid, push_threads<R>(), sm, st>>>(K, h, p, g, table, cnt, tv, so, ko);
+    launch_push_mode<R, NS, kPushSort>(K, h, p, g, table, cnt, tv, cap, sm_count, st, so, ko);
   else if (ko.keys)
-    k_push<R, NS, kPushKeys><<<grid, push_threads<R>(), sm, st>>>(K, h, p, g, table, cnt, tv, so, ko);
+    launch_push_mode<R, NS, kPushKeys>(K, h, p, g, table, cnt, tv, cap, sm_count, st, so, ko);
   else
-    k_push<R, NS, kPushPlain><<<grid, push_threads<R>(), sm, st>>>(K, h, p, g, table, cnt, tv, so, ko);
+    launch_push_mode<R, NS, kPushPlain>(K, h, p, g, table, cnt, tv, cap, sm_count, st, so, ko);
 }
 
 template <typename R>
 void launch_push(const Consts &K, PView<R> p, GView<R> g, const R *table, Counters *cnt,
-                 TallyView tv, int grid, cudaStream_t st, const SortOut<R> &so,
-                 const KeyOut<R> &ko) {
+                 TallyView tv, long long cap, int sm_count, cudaStream_t st,
+                 const SortOut<R> &so, const KeyOut<R> &ko) {
   const HotK<R> h = make_hot<R>(K);
   if (K.n_solids == 1)  // a single-element solid: the element loops vanish
-    launch_push_ns<R, 1>(K, h, p, g, table, cnt, tv, grid, st, so, ko);
+    launch_push_ns<R, 1>(K, h, p, g, table, cnt, tv, cap, sm_count, st, so, ko);
   else
-    launch_push_ns<R, 4>(K, h, p, g, table, cnt, tv, grid, st, so, ko);
+    launch_push_ns<R, 4>(K, h, p, g, table, cnt, tv, cap, sm_count, st, so, ko);
 }
 
 template <typename R>
@@ -281,10 +303,10 @@ void launch_advance(Counters *cnt, long long cap, cudaStream_t st) {
 }
 
 template void launch_push<float>(const Consts &, PView<float>, GView<float>, const float *,
-                                 Counters *, TallyView, int, cudaStream_t, const SortOut<float> &,
-                                 const KeyOut<float> &);
+                                 Counters *, TallyView, long long, int, cudaStream_t,
+                                 const SortOut<float> &, const KeyOut<float> &);
 template void launch_push<double>(const Consts &, PView<double>, GView<double>, const double *,
-                                  Counters *, TallyView, int, cudaStream_t,
+                                  Counters *, TallyView, long long, int, cudaStream_t,
                                   const SortOut<double> &, const KeyOut<double> &);
 template void launch_inject<float>(const Consts &, PView<float>, Counters *, long long, TallyView,
                                    int, cudaStream_t);
