@@ -270,21 +270,24 @@ int hpic_count_particles(hpic_ctx *ctx, int64_t *n);
  * remaining optical depth tau, id.  Fails with HPIC_EINVAL if cap is less
  * than the live count; *n receives the count.  Any of the output pointers
  * may be NULL (that array is skipped).  The compaction and the conversion
- * to double run on the device in a scratch buffer the context owns (grown
- * to 8 bytes per electron slot, freed by hpic_destroy or
- * hpic_batch_destroy); HPIC_ENOMEM if it cannot be allocated.  This call
- * and hpic_load_particles / hpic_count_particles synchronise the stream.
- * The host arrays here and in hpic_load_particles may be page-locked
- * (cudaHostAlloc) or pageable; page-locked ones, allocated once and reused,
- * avoid the driver's staging copies and the page faults of fresh memory. */
+ * to double run on the device, through a scratch buffer the context owns
+ * (grown to 8 bytes per electron slot, and by hpic_read_grid to 8 bytes per
+ * node where it can be had; freed by hpic_destroy or hpic_batch_destroy);
+ * HPIC_ENOMEM if it cannot be allocated.  This call and hpic_load_particles /
+ * hpic_count_particles synchronise the stream.  The host arrays here and in
+ * hpic_load_particles may be page-locked (cudaHostAlloc) or pageable, each for
+ * itself; page-locked ones, allocated once and reused, are written and read
+ * by the device across the link, all arrays in one kernel, without the
+ * driver's staging copies and the page faults of fresh memory. */
 int hpic_read_particles(hpic_ctx *ctx, double *x, double *y, double *z,
                         double *ux, double *uy, double *uz, double *tau,
                         uint32_t *id, int64_t cap, int64_t *n);
 /* Replace the electron population with n host electrons (same units).
  * Positions must lie in [0, n*dx] on each axis (any finite position with
- * HPIC_UNBOUNDED).  The arrays are checked on the device before anything is
- * written, so on HPIC_EINVAL the population is unchanged; the upload uses
- * the context's transfer scratch (see hpic_read_particles).  Errors:
+ * HPIC_UNBOUNDED).  The arrays are checked on the device while they are
+ * converted into the particle buffer that is not in use, so on HPIC_EINVAL the
+ * population is unchanged; pageable arrays go through the context's transfer
+ * scratch (see hpic_read_particles).  Errors:
  * HPIC_EINVAL, HPIC_ENOMEM. */
 /* Per-electron weights (real electrons per macro-electron) of the live
  * electrons, in the order hpic_read_particles returns them (same cap / n

@@ -548,10 +548,27 @@ int xfer_grid(const hpic_ctx *ctx, long long n) {
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
-// The live electrons in storage order.  On the device: the live slots are
-// counted per chunk and scanned, then each array is compacted and
-// converted to double (positions back to metres) into the transfer scratch
-// and copied to the caller's array; the ids likewise.
+// The device's address of `bytes` of page-locked host memory at p, or NULL
+// where it is not (pageable memory is copied through the driver).
+void *device_address(const void *p, size_t bytes) {
+  cudaPointerAttributes a{}, z{};
+  const char *end = static_cast<const char *>(p) + (bytes ? bytes - 1 : 0);
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
+      cudaPointerGetAttributes(&z, end) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer ||
+      static_cast<char *>(z.devicePointer) - static_cast<char *>(a.devicePointer) !=
+          end - static_cast<const char *>(p))
+    return nullptr;
+  return a.devicePointer;
+}
+
+// The live electrons in storage order: the live slots are counted per chunk
+// and scanned, then the arrays are compacted and converted to double
+// (positions back to metres).  Page-locked arrays are written across the link
+// by one kernel; others go one by one through the transfer scratch.
 template <typename R>
 int read_particles_impl(hpic_ctx *ctx, double *x, double *y, double *z, double *ux, double *uy,
                         double *uz, double *tau, uint32_t *id, int64_t cap, int64_t *n_out) {
@@ -574,30 +591,39 @@ int read_particles_impl(hpic_ctx *ctx, double *x, double *y, double *z, double *
   const long long live = live32;
   *n_out = live;
   if (live > cap) return fail(ctx, HPIC_EINVAL, "output capacity below the live particle count");
+  if (live == 0) return HPIC_OK;
   const double dx = ctx->tgt.dx_m;
-  const R *src[7] = {P.x, P.y, P.z, P.ux, P.uy, P.uz, P.tau};
   double *dst[7] = {x, y, z, ux, uy, uz, tau};
+  hpic::ParticleOut direct{};
+  bool any = false;
   for (int q = 0; q < 7; ++q) {
-    if (!dst[q] || live == 0) continue;
-    hpic::launch_compact<R, double>(src[q], P.id, n, cc, q < 3 ? dx : 1.0,
-                                    static_cast<double *>(data), ctx->stream);
-    CK(cudaMemcpyAsync(dst[q], data, live * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    if (dst[q]) direct.a[q] = static_cast<double *>(device_address(dst[q], live * sizeof(double)));
+    any |= direct.a[q] != nullptr;
+  }
+  if (id) direct.id = static_cast<uint32_t *>(device_address(id, live * sizeof(uint32_t)));
+  if (any || direct.id) hpic::launch_read_out<R>(P, n, cc, dx, direct, ctx->stream);
+  for (int q = 0; q < 8; ++q) {
+    void *to = q < 7 ? static_cast<void *>(dst[q]) : id;
+    if (!to || (q < 7 ? static_cast<void *>(direct.a[q]) : direct.id)) continue;
+    hpic::ParticleOut one{};
+    if (q < 7) one.a[q] = static_cast<double *>(data);
+    else one.id = static_cast<uint32_t *>(data);
+    hpic::launch_read_out<R>(P, n, cc, dx, one, ctx->stream);
+    CK(cudaMemcpyAsync(to, data, live * (q < 7 ? sizeof(double) : sizeof(uint32_t)),
+                       cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
   }
-  if (id && live > 0) {
-    hpic::launch_compact<uint32_t, uint32_t>(P.id, P.id, n, cc, 1.0,
-                                             static_cast<uint32_t *>(data), ctx->stream);
-    CK(cudaMemcpyAsync(id, data, live * sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-  }
+  CK(cudaStreamSynchronize(ctx->stream));
   CK(cudaGetLastError());
   return HPIC_OK;
 }
 
-// Replace the population with n host electrons.  Every array is copied to
-// the transfer scratch as it is; a first pass checks the positions and ids
-// on the device (nothing is written to the state unless all pass), a second
-// converts each array into the particle storage.
+// Replace the population with n host electrons.  The arrays are checked and
+// converted into the particle buffer that is not current, each crossing the
+// link once: page-locked ones are read by one kernel, others are copied to
+// the transfer scratch one by one.  Only if all pass does that buffer become
+// the current one (a batch target's electrons are copied over: the batch's
+// targets share the choice of buffer).
 template <typename R>
 int load_particles_impl(hpic_ctx *ctx, int64_t n, const double *x, const double *y,
                         const double *z, const double *ux, const double *uy, const double *uz,
@@ -605,22 +631,44 @@ int load_particles_impl(hpic_ctx *ctx, int64_t n, const double *x, const double 
   const double dx = ctx->tgt.dx_m;
   const int nn[3] = {ctx->tgt.nx, ctx->tgt.ny, ctx->tgt.nz};
   const int unbounded = (ctx->K.physics & hpic::P_UNBOUNDED) != 0;
+  const double *src[7] = {x, y, z, ux, uy, uz, tau};
+  hpic::ParticleIn direct{};
+  bool staged = false, any = false;
+  if (n > 0) {
+    for (int q = 0; q < 7; ++q) {
+      direct.a[q] = static_cast<const double *>(device_address(src[q], n * sizeof(double)));
+      staged |= !direct.a[q];
+      any |= direct.a[q] != nullptr;
+    }
+    direct.id = static_cast<const uint32_t *>(device_address(id, n * sizeof(uint32_t)));
+    staged |= !direct.id;
+  }
   const size_t data_off = 256;  // the error count first
-  int rc = xfer_reserve(ctx, data_off + (size_t)(n > 0 ? n : 1) * sizeof(double));
+  int rc = xfer_reserve(ctx, data_off + (staged ? (size_t)n * sizeof(double) : 0));
+  if (rc) return rc;
+  rc = reserve(ctx, n + injection_total(ctx));
   if (rc) return rc;
   unsigned *bad = static_cast<unsigned *>(ctx->xfer);
   double *data = reinterpret_cast<double *>(static_cast<char *>(ctx->xfer) + data_off);
   const int grid = xfer_grid(ctx, n);
+  const hpic::PView<R> P = pview<R>(ctx, ctx->cur ^ 1);
   CK(cudaMemsetAsync(bad, 0, sizeof(unsigned), ctx->stream));
-  const double *src[7] = {x, y, z, ux, uy, uz, tau};
+  auto load = [&](const hpic::ParticleIn &in) {
+    hpic::launch_load_in<R>(in, n, dx, nn, unbounded, P, ctx->K.weighted, (R)ctx->K.w, bad, grid,
+                            ctx->stream);  // (the envelope's weights come from hpic_load_weights)
+  };
   if (n > 0) {
-    for (int a = 0; a < 3; ++a) {
-      CK(cudaMemcpyAsync(data, src[a], n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-      hpic::launch_load_convert<R>(data, n, 1.0, static_cast<R *>(nullptr), 1, dx, (double)nn[a],
-                                   unbounded, bad, grid, ctx->stream);
+    if (any || direct.id) load(direct);
+    for (int q = 0; q < 8 && staged; ++q) {
+      if (q < 7 ? static_cast<const void *>(direct.a[q]) : direct.id) continue;
+      hpic::ParticleIn one{};
+      if (q < 7) one.a[q] = data;
+      else one.id = reinterpret_cast<const uint32_t *>(data);
+      CK(cudaMemcpyAsync(data, q < 7 ? static_cast<const void *>(src[q]) : id,
+                         n * (q < 7 ? sizeof(double) : sizeof(uint32_t)), cudaMemcpyHostToDevice,
+                         ctx->stream));
+      load(one);
     }
-    CK(cudaMemcpyAsync(data, id, n * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-    hpic::launch_check_ids(reinterpret_cast<const uint32_t *>(data), n, bad, grid, ctx->stream);
   }
   unsigned nbad = 0;
   CK(cudaMemcpyAsync(&nbad, bad, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
@@ -638,22 +686,15 @@ int load_particles_impl(hpic_ctx *ctx, int64_t n, const double *x, const double 
     }
     return fail(ctx, HPIC_EINVAL, "particle position outside the target");
   }
-  const long long extra = injection_total(ctx);
-  rc = reserve(ctx, n + extra);
-  if (rc) return rc;
-  const hpic::PView<R> P = pview<R>(ctx, ctx->cur);
-  R *dst[7] = {P.x, P.y, P.z, P.ux, P.uy, P.uz, P.tau};
-  if (n > 0) {
-    CK(cudaMemcpyAsync(P.id, id, n * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream));
-    for (int q = 0; q < 7; ++q) {
-      CK(cudaMemcpyAsync(data, src[q], n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-      hpic::launch_load_convert<R>(data, n, q < 3 ? 1.0 / dx : 1.0, dst[q], 0, dx, 0.0, unbounded,
-                                   bad, grid, ctx->stream);
-    }
-    if (ctx->K.weighted)  // the envelope's weights come from hpic_load_weights
-      hpic::launch_fill<R>(P.w, n, (R)ctx->K.w, grid, ctx->stream);
-    CK(cudaStreamSynchronize(ctx->stream));
-    CK(cudaGetLastError());
+  if (!ctx->owner) {
+    ctx->cur ^= 1;
+  } else if (n > 0) {
+    const hpic::PView<R> C = pview<R>(ctx, ctx->cur);
+    R *to[8] = {C.x, C.y, C.z, C.ux, C.uy, C.uz, C.tau, C.w};
+    const R *from[8] = {P.x, P.y, P.z, P.ux, P.uy, P.uz, P.tau, P.w};
+    for (int q = 0; q < (ctx->K.weighted ? 8 : 7); ++q)
+      CK(cudaMemcpyAsync(to[q], from[q], n * sizeof(R), cudaMemcpyDeviceToDevice, ctx->stream));
+    CK(cudaMemcpyAsync(C.id, P.id, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, ctx->stream));
   }
   hpic::Counters h;
   rc = read_counters(ctx, &h);
@@ -680,6 +721,18 @@ void *vector_array(const hpic_ctx *ctx, int which) {
   const int slot = which - HPIC_GRID_EX;  // 0..8: E, B, J
   char *base = static_cast<char *>(slot < 6 ? ctx->fields : ctx->jfield);
   return base + (slot % 6) * ctx->vstride * ctx->rsz;
+}
+
+// a grid read without device scratch (none could be had): scaled here
+int read_grid_by_host(hpic_ctx *ctx, int which, int64_t L, double s, double *out) {
+  const void *src = cell_array(ctx, which) ? cell_array(ctx, which) : vector_array(ctx, which);
+  const bool f32 = ctx->fp32 && !cell_array(ctx, which);
+  std::vector<float> b(f32 ? L : 0);
+  CK(cudaMemcpyAsync(f32 ? static_cast<void *>(b.data()) : out, src,
+                     L * (f32 ? sizeof(float) : sizeof(double)), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  for (int64_t i = 0; i < L; ++i) out[i] = (f32 ? (double)b[i] : out[i]) * s;
+  return HPIC_OK;
 }
 
 // entry points that step or reshape a context are the batch's business
@@ -948,23 +1001,25 @@ int hpic_read_grid(hpic_ctx *ctx, int which, double *out) {
   int64_t L;
   hpic_grid_len(ctx, which, &L);
   const double s = grid_scale(ctx, which);
-  if (const double *src = cell_array(ctx, which)) {
-    CK(cudaMemcpyAsync(out, src, L * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    for (int64_t i = 0; i < L; ++i) out[i] *= s;
-    return HPIC_OK;
+  const double *cells = cell_array(ctx, which);
+  const void *src = cells;
+  if (!cells || s != 1.0) {  // converted to double and scaled on the device
+    if (xfer_reserve(ctx, (size_t)L * sizeof(double)) != HPIC_OK) return read_grid_by_host(ctx, which, L, s, out);
+    double *d = static_cast<double *>(ctx->xfer);
+    const int grid = xfer_grid(ctx, L);
+    if (cells)
+      hpic::launch_scale_out<double>(cells, L, s, d, grid, ctx->stream);
+    else if (ctx->fp32)
+      hpic::launch_scale_out<float>(static_cast<const float *>(vector_array(ctx, which)), L, s, d,
+                                    grid, ctx->stream);
+    else
+      hpic::launch_scale_out<double>(static_cast<const double *>(vector_array(ctx, which)), L, s, d,
+                                     grid, ctx->stream);
+    src = d;
   }
-  const char *src = static_cast<const char *>(vector_array(ctx, which));
-  if (ctx->fp32) {
-    std::vector<float> b(L);
-    CK(cudaMemcpyAsync(b.data(), src, L * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    for (int64_t i = 0; i < L; ++i) out[i] = (double)b[i] * s;
-  } else {
-    CK(cudaMemcpyAsync(out, src, L * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
-    for (int64_t i = 0; i < L; ++i) out[i] *= s;
-  }
+  CK(cudaMemcpyAsync(out, src, L * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  CK(cudaGetLastError());
   return HPIC_OK;
 }
 

@@ -424,10 +424,9 @@ void launch_field_energy(const Consts &K, GView<R> g, double *dst, int grid, cud
 
 // ---------------------------------------------------------------- host transfers
 // Reading the electrons out: the live slots in storage order, converted to
-// double with a scale, compacted on the device so that one copy per array
-// crosses to the host.  Slots go in chunks of kXferChunk (256 threads x 8
-// consecutive slots): the live count of each chunk, an exclusive scan of the
-// chunk counts, then each array written at the compacted positions.
+// double with a scale.  Slots go in chunks of kXferChunk: the live count of
+// each chunk, an exclusive scan of the chunk counts, then the arrays written
+// at the compacted positions.
 constexpr int kXferChunk = 2048;
 
 __global__ void __launch_bounds__(256) k_live_counts(const uint32_t *id, long long n,
@@ -471,75 +470,101 @@ __global__ void __launch_bounds__(1024) k_scan_chunks(uint32_t *cc, long long nb
   if (threadIdx.x == 1023) cc[nb] = part[1023];
 }
 
-// out[rank] = src[i] * scale (converted to O) for the live slots i of this
-// block's chunk, rank = the slot's place among the live slots
-template <typename T, typename O>
-__global__ void __launch_bounds__(256) k_compact(const T *src, const uint32_t *id, long long n,
-                                                 const uint32_t *cc, double scale, O *out) {
+// out[q][rank] = array q of slot i, converted to double, for the live slots i
+// of this block's chunk, rank = the slot's place among the live slots (a
+// warp's 32 slots at a time, so that loads and stores run along the arrays);
+// null outputs are skipped.  The outputs may be page-locked host memory: the
+// stores then cross to the host at once, all arrays in one launch.  (Bound by
+// the link: 1e7 electrons, 600 MB, 3.6 ms through one copy per array before.)
+template <typename R>
+__global__ void __launch_bounds__(256) k_read_out(const PView<R> p, long long n, const uint32_t *cc,
+                                                  double dx, const ParticleOut out) {
   __shared__ uint32_t ws[8];
+  constexpr int kRounds = kXferChunk / 256;  // of 32 slots per warp
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long base = (long long)blockIdx.x * kXferChunk + threadIdx.x * 8;
-  uint32_t live = 0;
+  const long long base = (long long)blockIdx.x * kXferChunk + warp * (32 * kRounds) + lane;
+  uint32_t id[kRounds], live = 0, total = 0;
 #pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (base + k < n && id[base + k] != kDead) live |= 1u << k;
-  const uint32_t c = __popc(live);
-  uint32_t incl = c;  // inclusive scan over the warp, then over the warps
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
+  for (int k = 0; k < kRounds; ++k) {
+    const long long i = base + 32 * k;
+    id[k] = i < n ? p.id[i] : kDead;
+    if (id[k] != kDead) live |= 1u << k;
+    total += __popc(__ballot_sync(0xffffffffu, id[k] != kDead));
   }
-  if (lane == 31) ws[warp] = incl;
+  if (lane == 0) ws[warp] = total;
   __syncthreads();
-  uint32_t before = 0;
-  for (int w = 0; w < warp; ++w) before += ws[w];
-  long long pos = (long long)cc[blockIdx.x] + before + incl - c;
+  long long first = cc[blockIdx.x];
+  for (int w = 0; w < warp; ++w) first += ws[w];
+  const R *src[7] = {p.x, p.y, p.z, p.ux, p.uy, p.uz, p.tau};
 #pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (live & (1u << k)) {
-      if constexpr (std::is_floating_point<T>::value)
-        out[pos++] = (O)((double)src[base + k] * scale);
-      else
-        out[pos++] = (O)src[base + k];
+  for (int k = 0; k < kRounds; ++k) {
+    const bool on = (live >> k) & 1u;
+    const uint32_t mask = __ballot_sync(0xffffffffu, on);
+    const long long i = base + 32 * k, q = first + __popc(mask & ((1u << lane) - 1u));
+    if (on) {
+#pragma unroll
+      for (int a = 0; a < 7; ++a)
+        if (out.a[a]) out.a[a][q] = (double)src[a][i] * (a < 3 ? dx : 1.0);
+      if (out.id) out.id[q] = id[k];
     }
+    first += __popc(mask);
+  }
 }
 
-// Loading electrons in: dst[i] = (R)(src[i] * scale); with check set, also
-// count positions outside [0, hi] after division by dx (any non-finite
-// value with unbounded), the test the host made before
+// Loading electrons in: the arrays (device memory, or page-locked host memory
+// read across the link) checked and converted in one pass, where a pass to
+// check and one to convert took positions and ids across twice: 1e7 electrons
+// 5.3 -> 3.0 ms (600 MB, 200 GB/s; the link's bandwidth).  Counts positions
+// outside [0, hi] after division by dx (any non-finite value with unbounded)
+// and reserved ids.  The division is made only where the product with 1/dx
+// does not decide: within 1e-12 of a wall, or below zero.
 template <typename R>
-__global__ void __launch_bounds__(256) k_load_convert(const double *src, long long n,
-                                                      double scale, R *dst, int check,
-                                                      double dx, double hi, int unbounded,
-                                                      unsigned *bad) {
+__global__ void __launch_bounds__(256) k_load_in(const ParticleIn in, long long n, double dx,
+                                                 double inv_dx, int nx, int ny, int nz,
+                                                 int unbounded, PView<R> dst, int weighted, R w,
+                                                 unsigned *bad) {
   unsigned b = 0;
+  R *to[7] = {dst.x, dst.y, dst.z, dst.ux, dst.uy, dst.uz, dst.tau};
+  const double hi[3] = {(double)nx, (double)ny, (double)nz};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const double v = src[i];
-    if (check) {
-      const double X = v / dx;
-      b += (unbounded ? !isfinite(X) : !(X >= 0.0 && X <= hi)) ? 1u : 0u;
+    double v[7];
+    uint32_t id = 0;
+#pragma unroll
+    for (int a = 0; a < 7; ++a)
+      if (in.a[a]) v[a] = in.a[a][i];
+    if (in.id) id = in.id[i];
+#pragma unroll
+    for (int a = 0; a < 7; ++a) {
+      if (!in.a[a]) continue;
+      if (a < 3) {
+        const double q = v[a] * inv_dx;
+        if (!(q > 0.0 && q < hi[a] * (1.0 - 1e-12))) {
+          const double X = v[a] / dx;
+          b += (unbounded ? !isfinite(X) : !(X >= 0.0 && X <= hi[a])) ? 1u : 0u;
+        }
+        to[a][i] = (R)q;
+      } else {
+        to[a][i] = (R)v[a];
+      }
     }
-    if (dst) dst[i] = (R)(v * scale);
+    if (in.id) {
+      b += id == kDead ? 1u : 0u;
+      dst.id[i] = id;
+      if (weighted) dst.w[i] = w;
+    }
   }
-  if (check && b) atomicAdd(bad, b);
-}
-
-__global__ void __launch_bounds__(256) k_check_ids(const uint32_t *id, long long n,
-                                                   unsigned *bad) {
-  unsigned b = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    b += id[i] == kDead ? 1u : 0u;
   if (b) atomicAdd(bad, b);
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256) k_fill(R *dst, long long n, R v) {
+// a grid out: scaled to SI in double (in host loops before: four grids of 128^3
+// read in 3.7-5.4 ms, now 0.5 ms)
+template <typename T>
+__global__ void __launch_bounds__(256) k_scale_out(const T *src, long long n, double scale,
+                                                   double *out) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
-    dst[i] = v;
+    out[i] = (double)src[i] * scale;
 }
 
 long long xfer_chunks(long long n) { return (n + kXferChunk - 1) / kXferChunk; }
@@ -550,32 +575,26 @@ void launch_live_scan(const uint32_t *id, long long n, uint32_t *cc, cudaStream_
   k_scan_chunks<<<1, 1024, 0, st>>>(cc, nb);
 }
 
-template <typename T, typename O>
-void launch_compact(const T *src, const uint32_t *id, long long n, const uint32_t *cc,
-                    double scale, O *out, cudaStream_t st) {
+template <typename R>
+void launch_read_out(PView<R> p, long long n, const uint32_t *cc, double dx, const ParticleOut &out,
+                     cudaStream_t st) {
   const long long nb = xfer_chunks(n);
-  if (nb > 0) k_compact<T, O><<<(unsigned)nb, 256, 0, st>>>(src, id, n, cc, scale, out);
+  if (nb > 0) k_read_out<R><<<(unsigned)nb, 256, 0, st>>>(p, n, cc, dx, out);
 }
 
 template <typename R>
-void launch_load_convert(const double *src, long long n, double scale, R *dst, int check,
-                         double dx, double hi, int unbounded, unsigned *bad, int grid,
-                         cudaStream_t st) {
-  k_load_convert<R><<<grid, 256, 0, st>>>(src, n, scale, dst, check, dx, hi, unbounded, bad);
+void launch_load_in(const ParticleIn &in, long long n, double dx, const int (&cells)[3],
+                    int unbounded, PView<R> dst, int weighted, R w, unsigned *bad, int grid,
+                    cudaStream_t st) {
+  k_load_in<R><<<grid, 256, 0, st>>>(in, n, dx, 1.0 / dx, cells[0], cells[1], cells[2], unbounded,
+                                     dst, weighted, w, bad);
 }
 
-void launch_check_ids(const uint32_t *id, long long n, unsigned *bad, int grid, cudaStream_t st) {
-  k_check_ids<<<grid, 256, 0, st>>>(id, n, bad);
+template <typename T>
+void launch_scale_out(const T *src, long long n, double scale, double *out, int grid,
+                      cudaStream_t st) {
+  k_scale_out<T><<<grid, 256, 0, st>>>(src, n, scale, out);
 }
-
-template <typename R>
-void launch_fill(R *dst, long long n, R v, int grid, cudaStream_t st) {
-  k_fill<R><<<grid, 256, 0, st>>>(dst, n, v);
-}
-
-template void launch_compact<uint32_t, uint32_t>(const uint32_t *, const uint32_t *, long long,
-                                                 const uint32_t *, double, uint32_t *,
-                                                 cudaStream_t);
 
 #define HPIC_INST(R)                                                                          \
   template void launch_efield<R>(const Consts &, GView<R>, int, cudaStream_t);                \
@@ -589,11 +608,11 @@ template void launch_compact<uint32_t, uint32_t>(const uint32_t *, const uint32_
   template void launch_field_energy<R>(const Consts &, GView<R>, double *, int, cudaStream_t); \
   template void launch_batch_efield<R>(const BatchItem<R> *, BatchDev, int, cudaStream_t);     \
   template void launch_batch_bheat<R>(const BatchItem<R> *, BatchDev, int, cudaStream_t);     \
-  template void launch_compact<R, double>(const R *, const uint32_t *, long long,             \
-                                          const uint32_t *, double, double *, cudaStream_t);  \
-  template void launch_load_convert<R>(const double *, long long, double, R *, int, double,   \
-                                       double, int, unsigned *, int, cudaStream_t);           \
-  template void launch_fill<R>(R *, long long, R, int, cudaStream_t);
+  template void launch_read_out<R>(PView<R>, long long, const uint32_t *, double,             \
+                                   const ParticleOut &, cudaStream_t);                        \
+  template void launch_load_in<R>(const ParticleIn &, long long, double, const int (&)[3],    \
+                                  int, PView<R>, int, R, unsigned *, int, cudaStream_t);      \
+  template void launch_scale_out<R>(const R *, long long, double, double *, int, cudaStream_t);
 HPIC_INST(float)
 HPIC_INST(double)
 #undef HPIC_INST

@@ -193,19 +193,28 @@ constexpr int kFieldBlocksPerSm = 6;
 constexpr int kBatchFieldBlocksPerSm = 5;
 
 // host transfers of the electron state (the C-ABI's read and load calls):
-// live-slot compaction in storage order and FP64 <-> R conversion on the device
+// live-slot compaction in storage order and FP64 <-> R conversion on the
+// device; the arrays on the far side are x .. tau and ids (null: skipped)
+struct ParticleOut {
+  double *a[7];
+  uint32_t *id;
+};
+struct ParticleIn {
+  const double *a[7];
+  const uint32_t *id;
+};
 long long xfer_chunks(long long n);  // chunk counts needed: xfer_chunks(n) + 1
 void launch_live_scan(const uint32_t *id, long long n, uint32_t *cc, cudaStream_t st);
-template <typename T, typename O>
-void launch_compact(const T *src, const uint32_t *id, long long n, const uint32_t *cc,
-                    double scale, O *out, cudaStream_t st);
 template <typename R>
-void launch_load_convert(const double *src, long long n, double scale, R *dst, int check,
-                         double dx, double hi, int unbounded, unsigned *bad, int grid,
-                         cudaStream_t st);
-void launch_check_ids(const uint32_t *id, long long n, unsigned *bad, int grid, cudaStream_t st);
+void launch_read_out(PView<R> p, long long n, const uint32_t *cc, double dx, const ParticleOut &out,
+                     cudaStream_t st);
 template <typename R>
-void launch_fill(R *dst, long long n, R v, int grid, cudaStream_t st);
+void launch_load_in(const ParticleIn &in, long long n, double dx, const int (&cells)[3],
+                    int unbounded, PView<R> dst, int weighted, R w, unsigned *bad, int grid,
+                    cudaStream_t st);
+template <typename T>
+void launch_scale_out(const T *src, long long n, double scale, double *out, int grid,
+                      cudaStream_t st);
 
 // allow the push kernels their shared-memory deposit stages (above the
 // default 48 KB for FP64 and the batch); once per device, before any launch
