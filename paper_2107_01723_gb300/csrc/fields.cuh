@@ -9,59 +9,97 @@ namespace hpic {
 // (i, j, k) of node q.  The two divisions by the row and plane lengths go
 // through multiplications by rounded-up reciprocals (Granlund & Montgomery,
 // "Division by invariant integers using multiplication", PLDI 1994): exact for
-// the node counts here, below 2^31 (checked at creation).
+// the node counts here, below 2^29 (checked at creation).
 template <typename R>
-__device__ __forceinline__ void node_of(const FieldK<R> &K, long long q, int &i, int &j, int &k) {
-  const unsigned uq = (unsigned)q;
-  const unsigned kk = K.by_sz.quotient(uq), r = uq - kk * (unsigned)K.sz;
+__device__ __forceinline__ void node_of(const FieldK<R> &K, unsigned q, int &i, int &j, int &k) {
+  const unsigned kk = K.by_sz.quotient(q), r = q - kk * (unsigned)K.sz;
   const unsigned jj = K.by_sy.quotient(r);
   k = (int)kk;
   j = (int)jj;
   i = (int)(r - jj * (unsigned)K.sy);
 }
 
-// x^(-3/2) of an in_range x: an FP32 estimate y, then y (1 - e)^(-1/2) with
-// e = 1 - x^3 y^2 (about 1e-6) to second order, the next term being below
-// 1e-18: eight FP64 operations, where rsqrt(x) cubed takes about fourteen
-__device__ __forceinline__ double pow_m32(double x) {
+// Element at a byte offset.  Grids stay below 2^32 bytes per array (at most
+// 2^27 - 2 cells, so 3^3/2^3 as many nodes), and a 32-bit offset to a base that
+// is the same for all lanes takes one instruction less per access than a
+// 64-bit index: these kernels issue some thirty accesses per node.
+template <typename T>
+__device__ __forceinline__ T &at(T *p, unsigned off) {
+  return *reinterpret_cast<T *>(reinterpret_cast<char *>(p) + off);
+}
+template <typename T>
+__device__ __forceinline__ T at(const T *p, unsigned off) {
+  return *reinterpret_cast<const T *>(reinterpret_cast<const char *>(p) + off);
+}
+
+// r^2 of a positive normal r, exactly, in integers (24 x 24 bits)
+__device__ __forceinline__ double exact_square(float r) {
+  const unsigned b = __float_as_uint(r), m = (b & 0x007fffffu) | 0x00800000u;
+  const unsigned long long p = (unsigned long long)m * m;  // in [2^46, 2^48)
+  const unsigned top = (unsigned)(p >> 47);
+  const unsigned long long frac = p << (6 - top);  // leading one at bit 52
+  const unsigned exp = 2u * (b >> 23) + 769u + top;
+  return __longlong_as_double((long long)((frac & 0x000fffffffffffffull) |
+                                          ((unsigned long long)exp << 52)));
+}
+// c x^(-3/2) of an in_range x: r, an FP32 estimate of x^(-1/2), then c r^3
+// (1 + e)^(-3/2) with e = x r^2 - 1 (about 1e-7) to second order, the next term
+// being below 1e-19: six FP64 operations, where rsqrt(x) cubed takes about
+// fifteen
+__device__ __forceinline__ double times_pow_m32(double c, double x) {
   const float r = rsqrtf(narrow(x));
-  const double y = widen(r * r * r);
-  const double e = fma(-(x * x * x), y * y, 1.0);
-  return fma(y, e * fma(0.375, e, 0.5), y);
+  const double r2 = exact_square(r), e = fma(x, r2, -1.0);
+  const double s = c * r2 * widen(r);
+  return fma(s, e * fma(1.875, e, -1.5), s);
 }
 
 // ---------------------------------------------------------------- E, Eq. (A2)
 // E on the three edges owned by node q (tangential E = 0 on the walls)
 template <typename R>
-__device__ __forceinline__ void efield_node(const FieldK<R> &K, const GView<R> &g, long long q) {
+__device__ __forceinline__ void efield_node(const FieldK<R> &K, const GView<R> &g, unsigned node) {
+  constexpr unsigned Z = sizeof(R);
   const int nx = K.nx, ny = K.ny, nz = K.nz;
-  const int sy = K.sy;
-  const long long sz = K.sz;
-  const long long cy = nx, cz = (long long)nx * ny;
+  const unsigned q = node * Z, sy = K.sy * Z, sz = K.sz * Z;
+  const unsigned cy = nx * Z, cz = nx * ny * Z;
   const R Fc = K.F_curl, Fj = K.F_j;
-  const R *Bx = g.B[0], *By = g.B[1], *Bz = g.B[2];
+  const R *Bx = g.B[0], *By = g.B[1], *Bz = g.B[2], *eta = g.eta_r;
   int i, j, k;
-  node_of(K, q, i, j, k);
+  node_of(K, node, i, j, k);
   R ex = 0, ey = 0, ez = 0;
-  const long long c = i + cy * j + cz * k;  // cell (i, j, k)
-  if (i < nx && j >= 1 && j <= ny - 1 && k >= 1 && k <= nz - 1) {
-    const R curl = (Bz[q] - Bz[q - sy]) - (By[q] - By[q - sz]);
-    const R eta = R(0.25) * (g.eta_r[c - cy - cz] + g.eta_r[c - cz] + g.eta_r[c - cy] + g.eta_r[c]);
-    ex = eta * (Fc * curl - Fj * g.J[0][q]);
+  const unsigned c = (unsigned)(i + nx * (j + ny * k)) * Z;  // cell (i, j, k)
+  const bool in_i = i >= 1 && i < nx, in_j = j >= 1 && j < ny, in_k = k >= 1 && k < nz;
+  if (in_i && in_j && in_k) {
+    // away from the walls all three edges share their loads, which are issued
+    // together: the kernel lives on memory latency
+    const R bx = at(Bx, q), bxy = at(Bx, q - sy), bxz = at(Bx, q - sz);
+    const R by = at(By, q), byx = at(By, q - Z), byz = at(By, q - sz);
+    const R bz = at(Bz, q), bzx = at(Bz, q - Z), bzy = at(Bz, q - sy);
+    const R jx = at<const R>(g.J[0], q), jy = at<const R>(g.J[1], q), jz = at<const R>(g.J[2], q);
+    const R e0 = at(eta, c), ei = at(eta, c - Z), ej = at(eta, c - cy), ek = at(eta, c - cz);
+    const R eij = at(eta, c - Z - cy), eik = at(eta, c - Z - cz), ejk = at(eta, c - cy - cz);
+    ex = R(0.25) * (ejk + ek + ej + e0) * (Fc * ((bz - bzy) - (by - byz)) - Fj * jx);
+    ey = R(0.25) * (eik + ek + ei + e0) * (Fc * ((bx - bxz) - (bz - bzx)) - Fj * jy);
+    ez = R(0.25) * (eij + ej + ei + e0) * (Fc * ((by - byx) - (bx - bxy)) - Fj * jz);
+  } else {
+    if (i < nx && in_j && in_k) {
+      const R curl = (at(Bz, q) - at(Bz, q - sy)) - (at(By, q) - at(By, q - sz));
+      const R e = R(0.25) * (at(eta, c - cy - cz) + at(eta, c - cz) + at(eta, c - cy) + at(eta, c));
+      ex = e * (Fc * curl - Fj * at<const R>(g.J[0], q));
+    }
+    if (j < ny && in_i && in_k) {
+      const R curl = (at(Bx, q) - at(Bx, q - sz)) - (at(Bz, q) - at(Bz, q - Z));
+      const R e = R(0.25) * (at(eta, c - Z - cz) + at(eta, c - cz) + at(eta, c - Z) + at(eta, c));
+      ey = e * (Fc * curl - Fj * at<const R>(g.J[1], q));
+    }
+    if (k < nz && in_i && in_j) {
+      const R curl = (at(By, q) - at(By, q - Z)) - (at(Bx, q) - at(Bx, q - sy));
+      const R e = R(0.25) * (at(eta, c - Z - cy) + at(eta, c - cy) + at(eta, c - Z) + at(eta, c));
+      ez = e * (Fc * curl - Fj * at<const R>(g.J[2], q));
+    }
   }
-  if (j < ny && i >= 1 && i <= nx - 1 && k >= 1 && k <= nz - 1) {
-    const R curl = (Bx[q] - Bx[q - sz]) - (Bz[q] - Bz[q - 1]);
-    const R eta = R(0.25) * (g.eta_r[c - 1 - cz] + g.eta_r[c - cz] + g.eta_r[c - 1] + g.eta_r[c]);
-    ey = eta * (Fc * curl - Fj * g.J[1][q]);
-  }
-  if (k < nz && i >= 1 && i <= nx - 1 && j >= 1 && j <= ny - 1) {
-    const R curl = (By[q] - By[q - 1]) - (Bx[q] - Bx[q - sy]);
-    const R eta = R(0.25) * (g.eta_r[c - 1 - cy] + g.eta_r[c - cy] + g.eta_r[c - 1] + g.eta_r[c]);
-    ez = eta * (Fc * curl - Fj * g.J[2][q]);
-  }
-  g.E[0][q] = ex;
-  g.E[1][q] = ey;
-  g.E[2][q] = ez;
+  at(g.E[0], q) = ex;
+  at(g.E[1], q) = ey;
+  at(g.E[2], q) = ez;
 }
 
 // rho / (Z n_i k_B C(T)) with the heat capacity of Eq. (A8),
@@ -91,17 +129,17 @@ __device__ __forceinline__ R heat_increment(const FieldK<R> &K, R T, R rho) {
 // reduced Lee-More resistivity, Eqs. (A4)-(A6), capped; inside the band
 // where the cap holds, the cap itself.  eta_num / max(tau_hot, tau_cold) is
 // the smaller of eta_num/(A_hot (kT)^1.5) and eta_num sqrt(kT)/B_cold.
-// In range, both come from p = T^(-3/2) (sqrt(T) = T^2 p) without a division,
+// In range, both come from T^(-3/2) (sqrt(T) = T^2 T^(-3/2)) without a division,
 // a root or a compare on the FP64 unit (Tf = (float)T tells the band, whose
-// float ends lie inside the exact one, where the formula gives the cap too):
-// this and the conversions took the heating of 128^3 cells from 128 to 71 us,
-// and of a 16-target batch of 7.9e6 cells (each with its constants in shared
-// memory and its Ohmic sums made in the warp) from 542 to 199 us.
+// float ends lie inside the exact one, where the formula gives the cap too).
+// A heated cell took 29 FP64 instructions, the SM's FP64 unit a warp-wide one
+// in 19 clocks: 128 us for 128^3 cells, now 8 to 9 and 51 us; a batch of 7.9e6
+// cells (each target's constants in shared memory, its Ohmic sums made in the
+// warp) 542 -> 145 us.
 __device__ __forceinline__ double resistivity(const FieldCommon &K, double T, float Tf) {
   if (Tf > K.eta_Tlo && Tf < K.eta_Thi) return K.eta_max;
-  const double p = pow_m32(T);
-  double eta = K.eta_hot * p;
-  if (K.eta_cold > 0.0) eta = min_positive(eta, K.eta_cold * (T * T * p));
+  double eta = times_pow_m32(K.eta_hot, T);
+  if (K.cold) eta = min_positive(eta, times_pow_m32(K.eta_cold, T) * (T * T));
   return min_positive(eta, K.eta_max);
 }
 // the same for any T
@@ -116,43 +154,85 @@ inline __device__ __noinline__ double resistivity_any(double eta_hot, double eta
   return eta < eta_max ? eta : eta_max;
 }
 
+// F_sigma (App. B) of the ion temperature, for the FP32 push by an FP32
+// logarithm of the significand (below 0.35, error 3e-8) added in FP64 to the
+// exponent's: 5e-8 of the logarithm, times fs_q (below 1/4), which stays under
+// the rounding of the result
+template <typename R>
+__device__ __forceinline__ R fsigma(const FieldCommon &K, double Ti) {
+  double half_log;
+  if (sizeof(R) == 4 && in_range(Ti)) {
+    const unsigned b = __float_as_uint(narrow(Ti));
+    float m = __uint_as_float((b & 0x007fffffu) | 0x3f800000u);
+    int k = (int)(b >> 23) - 127;
+    if (m > 1.41421356f) {
+      m *= 0.5f;
+      ++k;
+    }
+    half_log = fma((double)k, 0.5 * 0.693147180559945309417232, 0.5 * (double)logf(m));
+  } else {
+    half_log = 0.5 * log(Ti);
+  }
+  return R(fma(K.fs_q, half_log + K.fs_c, 1.0));
+}
+
 // ---------------------------------------------------------------- B, Eq. (A3), and heating
 // Faraday on the faces owned by node q, then heating of cell q; the cell's
 // Ohmic energy density (J/m^3) goes to `ohm`
 template <typename R>
-__device__ __forceinline__ void bheat_node(const FieldK<R> &K, const GView<R> &g, long long q,
+__device__ __forceinline__ void bheat_node(const FieldK<R> &K, const GView<R> &g, unsigned node,
                                            WideSum<R> &ohm) {
+  constexpr unsigned Z = sizeof(R), D = sizeof(double);
   const int nx = K.nx, ny = K.ny, nz = K.nz;
-  const int sy = K.sy;
-  const long long sz = K.sz;
+  const unsigned q = node * Z, sy = K.sy * Z, sz = K.sz * Z;
   const R cdt = K.cdt;
   const R *Ex = g.E[0], *Ey = g.E[1], *Ez = g.E[2];
   int i, j, k;
-  node_of(K, q, i, j, k);
-  if (K.physics & P_FARADAY) {
-    if (j < ny && k < nz) g.B[0][q] -= cdt * ((Ez[q + sy] - Ez[q]) - (Ey[q + sz] - Ey[q]));
-    if (i < nx && k < nz) g.B[1][q] -= cdt * ((Ex[q + sz] - Ex[q]) - (Ez[q + 1] - Ez[q]));
-    if (i < nx && j < ny) g.B[2][q] -= cdt * ((Ey[q + 1] - Ey[q]) - (Ex[q + sy] - Ex[q]));
-  }
-  if (i < nx && j < ny && k < nz) {
-    const long long c = i + (long long)nx * (j + (long long)ny * k);
-    const double Hc = g.H[c];
-    R jb2 = R(0);
-    if (K.physics & P_FIELDS) {
+  node_of(K, node, i, j, k);
+  const bool in_i = i < nx, in_j = j < ny, in_k = k < nz, cell = in_i && in_j && in_k;
+  const unsigned c = (unsigned)(i + nx * (j + ny * k));
+  const bool faraday = (K.physics & P_FARADAY) != 0, ohmic = (K.physics & P_FIELDS) != 0;
+  // everything a node reads but T and eta, before its first store: one round
+  // trip to memory, where loads between the stores of B made four
+  double Hc = 0.0;
+  R jx = 0, jy = 0, jz = 0;
+  if (cell) {
+    Hc = at<const double>(g.H, c * D);
+    if (ohmic) {
       const R *Jx = g.J[0], *Jy = g.J[1], *Jz = g.J[2];
-      // cell-centred mean of the edge current in the field precision
-      const R jbx = R(0.25) * (Jx[q] + Jx[q + sy] + Jx[q + sz] + Jx[q + sy + sz]);
-      const R jby = R(0.25) * (Jy[q] + Jy[q + 1] + Jy[q + sz] + Jy[q + 1 + sz]);
-      const R jbz = R(0.25) * (Jz[q] + Jz[q + 1] + Jz[q + sy] + Jz[q + 1 + sy]);
-      jb2 = jbx * jbx + jby * jby + jbz * jbz;
+      jx = at(Jx, q) + at(Jx, q + sy) + at(Jx, q + sz) + at(Jx, q + sy + sz);
+      jy = at(Jy, q) + at(Jy, q + Z) + at(Jy, q + sz) + at(Jy, q + Z + sz);
+      jz = at(Jz, q) + at(Jz, q + Z) + at(Jz, q + sy) + at(Jz, q + Z + sy);
     }
+  }
+  if (faraday) {
+    if (cell) {
+      const R ex = at(Ex, q), exy = at(Ex, q + sy), exz = at(Ex, q + sz);
+      const R ey = at(Ey, q), eyx = at(Ey, q + Z), eyz = at(Ey, q + sz);
+      const R ez = at(Ez, q), ezx = at(Ez, q + Z), ezy = at(Ez, q + sy);
+      const R bx = at<const R>(g.B[0], q), by = at<const R>(g.B[1], q), bz = at<const R>(g.B[2], q);
+      at(g.B[0], q) = bx - cdt * ((ezy - ez) - (eyz - ey));
+      at(g.B[1], q) = by - cdt * ((exz - ex) - (ezx - ez));
+      at(g.B[2], q) = bz - cdt * ((eyx - ey) - (exy - ex));
+    } else {
+      if (in_j && in_k) at(g.B[0], q) -= cdt * ((at(Ez, q + sy) - at(Ez, q)) - (at(Ey, q + sz) - at(Ey, q)));
+      if (in_i && in_k) at(g.B[1], q) -= cdt * ((at(Ex, q + sz) - at(Ex, q)) - (at(Ez, q + Z) - at(Ez, q)));
+      if (in_i && in_j) at(g.B[2], q) -= cdt * ((at(Ey, q + Z) - at(Ey, q)) - (at(Ex, q + sy) - at(Ex, q)));
+    }
+  }
+  if (cell) {
+    // cell-centred mean of the edge current in the field precision
+    jx *= R(0.25);
+    jy *= R(0.25);
+    jz *= R(0.25);
+    const R jb2 = jx * jx + jy * jy + jz * jz;
     // a cell without drag heat or current keeps T and eta (and adds no
     // Ohmic energy) unless e-i equilibration moves it
     const bool no_heat = (__double_as_longlong(Hc) << 1) == 0;  // +0 or -0
     if (no_heat && jb2 == R(0) && !(K.physics & P_EI)) return;
-    double Te = g.T[c];
+    double Te = at<const double>(g.T, c * D);
     bool changed = false;
-    const R ro = g.eta_r[c] * K.F_ohm * jb2;
+    const R ro = at<const R>(g.eta_r, c * Z) * K.F_ohm * jb2;
     ohm.add(ro);
     R rho = ro;
     if (!no_heat) {
@@ -174,15 +254,29 @@ __device__ __forceinline__ void bheat_node(const FieldK<R> &K, const GView<R> &g
     // b = rate_i dt frozen, the gap d = T_e - T_i decays by exp(-(a + b)) and
     // b T_e + a T_i is kept
     if (K.physics & P_EI) {
-      double Ti = g.Ti[c];
-      const double d = Te - Ti;
-      const double a = K.ei_a / pow(Te * K.ei_mi + Ti * K.ei_me, 1.5), b = K.Zstar * a;
-      if (d != 0.0 && a + b > 0.0) {
-        const double f = expm1(-(a + b)) / (a + b);
+      double Ti = at<const double>(g.Ti, c * D);
+      const double d = Te - Ti, X = Te * K.ei_mi + Ti * K.ei_me;
+      // (1.4e5 aluminium cells with this and F_sigma: 60.7 -> 17.5 us by the
+      // power, the series and fsigma() in place of pow, expm1, a division and log)
+      const double a = in_range(X) ? times_pow_m32(K.ei_a, X) : K.ei_a / pow(X, 1.5);
+      const double b = K.Zstar * a, s = a + b;
+      if (d != 0.0 && s > 0.0) {
+        // (e^{-s} - 1)/s: its series up to s = 1/64 (remainder below 1e-17)
+        double f;
+        if (s < 0.015625) {
+          f = fma(s, -1.0 / 5040.0, 1.0 / 720.0);
+          f = fma(s, f, -1.0 / 120.0);
+          f = fma(s, f, 1.0 / 24.0);
+          f = fma(s, f, -1.0 / 6.0);
+          f = fma(s, f, 0.5);
+          f = fma(s, f, -1.0);
+        } else {
+          f = expm1(-s) / s;
+        }
         Te += a * d * f;
         Ti -= b * d * f;
-        g.Ti[c] = Ti;
-        if (K.physics & P_FSIGMA) g.Fsig[c] = R(1.0 + K.fs_q * (0.5 * log(Ti) + K.fs_c));
+        at(g.Ti, c * D) = Ti;
+        if (K.physics & P_FSIGMA) at(g.Fsig, c * Z) = fsigma<R>(K, Ti);
         changed = true;
       }
     }
@@ -193,9 +287,9 @@ __device__ __forceinline__ void bheat_node(const FieldK<R> &K, const GView<R> &g
       } else {
         e = resistivity_any(K.eta_hot, K.eta_cold, K.eta_max, Te);
       }
-      g.T[c] = Te;
-      g.eta[c] = e;
-      if constexpr (sizeof(R) == 4) g.eta_r[c] = in_range(e) ? narrow(e) : (float)e;
+      at(g.T, c * D) = Te;
+      at(g.eta, c * D) = e;
+      if constexpr (sizeof(R) == 4) at(g.eta_r, c * Z) = in_range(e) ? narrow(e) : (float)e;
     }
   }
 }

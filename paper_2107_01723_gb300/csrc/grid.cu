@@ -14,8 +14,7 @@ namespace hpic {
 
 template <typename R>
 __global__ void __launch_bounds__(256, kFieldBlocksPerSm) k_efield(const FieldK<R> K, GView<R> g) {
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < K.nvec;
-       q += (long long)gridDim.x * blockDim.x)
+  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < K.nvec; q += gridDim.x * blockDim.x)
     efield_node(K, g, q);
 }
 
@@ -26,8 +25,7 @@ k_bheat(const FieldK<R> K, GView<R> g, TallyView tv) {
   if (threadIdx.x == 0) sum = 0.0;
   __syncthreads();
   WideSum<R> ohm;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < K.nvec;
-       q += (long long)gridDim.x * blockDim.x)
+  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < K.nvec; q += gridDim.x * blockDim.x)
     bheat_node(K, g, q, ohm);
   ohm.over_warp();
   if ((threadIdx.x & 31) == 0 && ohm.value() != 0.0) atomicAdd(&sum, ohm.value());
@@ -77,7 +75,7 @@ k_batch_efield(const BatchItem<R> *items, BatchDev d) {
   int t = -1;
   for (long long w = blockIdx.x * 8ll + warp; w < N; w += gridDim.x * 8ll) {
     t = enter_target(hot[warp], items, npref_s, t, w);
-    const long long q = (w - npref_s[t]) * 32 + lane;
+    const unsigned q = (unsigned)(w - npref_s[t]) * 32u + lane;
     if (q < hot[warp].K.nvec) efield_node(hot[warp].K, hot[warp].g, q);
   }
 }
@@ -105,7 +103,7 @@ k_batch_bheat(const BatchItem<R> *items, BatchDev d) {
   for (long long w = blockIdx.x * 8ll + warp; w < N; w += gridDim.x * 8ll) {
     if (t >= 0 && npref_s[t + 1] <= w) flush();
     t = enter_target(hot[warp], items, npref_s, t, w);
-    const long long q = (w - npref_s[t]) * 32 + lane;
+    const unsigned q = (unsigned)(w - npref_s[t]) * 32u + lane;
     if (q < hot[warp].K.nvec) bheat_node(hot[warp].K, hot[warp].g, q, ohm);
   }
   if (t >= 0) flush();

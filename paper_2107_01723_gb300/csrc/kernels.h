@@ -102,8 +102,9 @@ inline Quotient make_quotient(uint32_t d) {  // d >= 2
 struct FieldCommon {
   int nx, ny, nz, sy, sz;  // sy, sz: nodes per row and plane
   int physics, n_solids;
+  int cold;                // lambda1 > 0: eta_cold limits eta
   Quotient by_sy, by_sz;
-  long long nvec;
+  unsigned nvec;
   double F_H, dx3;
   double eta_hot, eta_cold, eta_max;  // eta = min(eta_hot T^-1.5, eta_cold T^0.5, eta_max), T in K
   float eta_Tlo, eta_Thi;             // eta(T) is at its cap in this band
@@ -126,11 +127,12 @@ inline FieldK<R> make_field(const Consts &K) {
   f.n_solids = K.n_solids;
   f.by_sy = make_quotient((uint32_t)f.sy);
   f.by_sz = make_quotient((uint32_t)f.sz);
-  f.nvec = K.nvec;
+  f.nvec = (unsigned)K.nvec;
   f.F_H = K.F_H;
   f.dx3 = K.dx3;
   f.eta_hot = K.eta_hot_T;
   f.eta_cold = K.eta_cold_T;
+  f.cold = K.eta_cold_T > 0.0;
   f.eta_max = K.eta_max;
   // the exact band's ends moved inwards by more than a float's rounding
   f.eta_Tlo = (float)(K.eta_Tlo * (1.0 + 5e-7));
@@ -188,9 +190,12 @@ constexpr int push_threads(int mode) {
 }
 // resident 256-thread blocks per SM of the field and heating kernels (their
 // launch bounds); they are launched as one wave of sm_count times this many
-// blocks (grid-stride over the nodes), so no partial second wave trails
-constexpr int kFieldBlocksPerSm = 6;
-constexpr int kBatchFieldBlocksPerSm = 5;
+// blocks (grid-stride over the nodes), so no partial second wave trails.  Four
+// (64 registers) hold a node's loads all at once: against six (40 registers)
+// the heating of 128^3 cells took 63 for 69 us, the field solve 23 for 25 us;
+// three were level.
+constexpr int kFieldBlocksPerSm = 4;
+constexpr int kBatchFieldBlocksPerSm = 4;
 
 // host transfers of the electron state (the C-ABI's read and load calls):
 // live-slot compaction in storage order and FP64 <-> R conversion on the
