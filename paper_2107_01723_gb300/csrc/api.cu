@@ -399,7 +399,6 @@ void destroy_all(hpic_ctx *c) {
   cudaFree(c->Ti);
   cudaFree(c->Fsig);
   cudaFree(c->inj_cells);
-  cudaFree(c->H);
   cudaFree(c->tal);
   cudaFree(c->hist);
   cudaFree(c->history);
@@ -434,8 +433,9 @@ int step_impl(hpic_ctx *ctx, long long nsteps) {
   const bool grid_on = !(ctx->K.physics & hpic::P_UNBOUNDED);
   for (long long s = 0; s < nsteps; ++s) {
     if (grid_on) {
-      CK(cudaMemsetAsync(G.J[0], 0, 3 * ctx->vstride * ctx->rsz, ctx->stream));
-      CK(cudaMemsetAsync(ctx->H, 0, ctx->K.ncell * sizeof(double), ctx->stream));
+      // the current and, behind it, the drag heat
+      CK(cudaMemsetAsync(G.J[0], 0, 3 * ctx->vstride * ctx->rsz + ctx->K.ncell * sizeof(double),
+                         ctx->stream));
     }
     // every sort_interval steps the cell sort rides on the step: its keys
     // come from the start-of-step state one step further ahead, and the push
@@ -489,28 +489,29 @@ int step_impl(hpic_ctx *ctx, long long nsteps) {
       ctx->ev_used += 2;
       ctx->prof_launches += 1;
     }
+    // a sort keeps the electrons before the dead bin's exclusive offset
+    const hpic::StepEnd end{ctx->cnt, sort_now ? ctx->counts + ctx->K.nkeys : nullptr, ctx->cap};
     if (grid_on && (ctx->K.physics & hpic::P_FIELDS)) {
       hpic::launch_efield<R>(ctx->K, G, gg, ctx->stream);
       ctx->launches += 1;
     }
     if (grid_on) {
-      hpic::launch_bheat<R>(ctx->K, G, tv, gg, ctx->stream);
+      hpic::launch_bheat<R>(ctx->K, G, tv, inject_now ? hpic::StepEnd{} : end, gg, ctx->stream);
       ctx->launches += 1;
     }
-    if (sort_now) {  // the kept electrons now fill the front of the other buffer
-      ctx->launches += hpic::launch_sort_finish(ctx->K, ctx->cnt, ctx->counts, ctx->stream);
-      ctx->cur ^= 1;
-    }
+    if (sort_now) ctx->cur ^= 1;  // the kept electrons fill the front of the other buffer
     if (inject_now) {
       const long long S = ctx->K.n_inj_steps, N = ctx->K.n_macro, st = ctx->host_step;
       const long long c = ctx->K.weighted ? ctx->K.per_cell * ctx->K.n_inj_cells
                                           : (N * (st + 1)) / S - (N * st) / S;
-      hpic::launch_inject<R>(ctx->K, P(ctx->cur), ctx->cnt, ctx->cap, tv,
-                             grid_blocks(ctx, c > 0 ? c : 1), ctx->stream);
+      hpic::launch_inject<R>(ctx->K, P(ctx->cur), end, tv, grid_blocks(ctx, c > 0 ? c : 1),
+                             ctx->stream);
       ctx->launches += 1;
     }
-    hpic::launch_advance(ctx->cnt, ctx->cap, ctx->stream);
-    ctx->launches += 1;
+    if (inject_now || !grid_on) {
+      hpic::launch_advance(end, ctx->stream);
+      ctx->launches += 1;
+    }
     ctx->host_step += 1;
     CK(cudaGetLastError());
   }
@@ -779,13 +780,13 @@ int hpic_init_target(hpic_ctx **out, const hpic_target_desc *t, const hpic_run_p
   const hpic::Consts &K = ctx->K;
   ctx->vstride = round_up(K.nvec + 4, 64);
   const long long m = K.nkeys + 1;
-  bool ok = cudaMalloc(&ctx->fields, 9 * ctx->vstride * ctx->rsz) == cudaSuccess &&
+  bool ok = cudaMalloc(&ctx->fields, 9 * ctx->vstride * ctx->rsz + K.ncell * sizeof(double)) ==
+                cudaSuccess &&
             cudaMalloc(&ctx->T, K.ncell * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&ctx->eta, K.ncell * sizeof(double)) == cudaSuccess &&
             (!ctx->fp32 || cudaMalloc(&ctx->eta_r, K.ncell * sizeof(float)) == cudaSuccess) &&
             cudaMalloc(&ctx->Ti, K.ncell * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&ctx->Fsig, K.ncell * ctx->rsz) == cudaSuccess &&
-            cudaMalloc(&ctx->H, K.ncell * sizeof(double)) == cudaSuccess &&
             cudaMalloc(&ctx->counts, m * sizeof(uint32_t)) == cudaSuccess &&
             cudaMalloc(&ctx->partials, hpic::scan_partials(m) * sizeof(uint32_t)) == cudaSuccess &&
             cudaMalloc(&ctx->tal, hpic::T_COUNT * sizeof(double)) == cudaSuccess &&
@@ -801,6 +802,7 @@ int hpic_init_target(hpic_ctx **out, const hpic_target_desc *t, const hpic_run_p
     return bail(HPIC_ENOMEM);
   }
   ctx->jfield = static_cast<char *>(ctx->fields) + 6 * ctx->vstride * ctx->rsz;
+  ctx->H = reinterpret_cast<double *>(static_cast<char *>(ctx->fields) + 9 * ctx->vstride * ctx->rsz);
   int rc = reserve(ctx, 1024);
   if (rc) return bail(rc);
   cudaStream_t st = ctx->stream;

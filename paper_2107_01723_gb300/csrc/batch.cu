@@ -45,8 +45,6 @@ struct hpic_batch {
   long long slots = 0;  // elements per particle array (all targets)
   void *jall = nullptr;
   size_t jall_bytes = 0;
-  double *hall = nullptr;
-  long long cells = 0;
   // per-step scratch, constants and tables: a second allocation
   void *aux = nullptr;
   void *items = nullptr;  // BatchItem<R>[n]
@@ -141,8 +139,7 @@ int enqueue_step(hpic_batch *b, bool sort) {
                                           (long long)b->sm_count * hpic::kBatchFieldBlocksPerSm);
   int k = 0;
   if (grid_on) {
-    BCK(cudaMemsetAsync(b->jall, 0, b->jall_bytes, b->stream));
-    BCK(cudaMemsetAsync(b->hall, 0, b->cells * sizeof(double), b->stream));
+    BCK(cudaMemsetAsync(b->jall, 0, b->jall_bytes, b->stream));  // current, then drag heat
   }
   hpic::launch_batch_plan<R>(items, b->d, b->stream);
   ++k;
@@ -183,12 +180,11 @@ int enqueue_step(hpic_batch *b, bool sort) {
     hpic::launch_batch_bheat<R>(items, b->d, gg, b->stream);
     ++k;
   }
-  if (sort) k += hpic::launch_batch_sort_finish<R>(items, b->d, b->stream);
   if (b->any_inject) {
-    hpic::launch_batch_inject<R>(items, b->d, Pnext, b->sm_count * 2, b->stream);
+    hpic::launch_batch_inject<R>(items, b->d, Pnext, sort, b->sm_count * 2, b->stream);
     ++k;
   }
-  hpic::launch_batch_advance<R>(items, b->d, b->stream);
+  hpic::launch_batch_advance<R>(items, b->d, sort, b->stream);
   ++k;
   BCK(cudaGetLastError());
   return k;
@@ -410,11 +406,10 @@ int hpic_batch_init(hpic_batch **out, int32_t n_targets, const hpic_target_desc 
     return bail(HPIC_EINVAL);
   }
   b->slots = slots;
-  b->cells = cells;
   b->nodes_total = 32 * npref[n_targets];
   b->nkeys_total = kpref[n_targets];
 
-  // arena: particles (x2), E and B, J, T, eta, heat, tallies, histograms,
+  // arena: particles (x2), E and B, J, heat, T, eta, tallies, histograms,
   // histories, counters, read scratch
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -424,9 +419,10 @@ int hpic_batch_init(hpic_batch **out, int32_t n_targets, const hpic_target_desc 
   };
   const size_t pb = (size_t)slots * (8 * b->rsz + sizeof(uint32_t));
   const size_t o_p0 = take(pb), o_p1 = take(pb);
-  const size_t o_eb = take(eb * b->rsz), o_j = take(jv * b->rsz);
+  const size_t o_eb = take(eb * b->rsz);
+  // the current and the drag heat side by side: cleared together every step
+  const size_t o_j = take(jv * b->rsz), o_H = take(cells * sizeof(double));
   const size_t o_T = take(cells * sizeof(double)), o_eta = take(cells * sizeof(double));
-  const size_t o_H = take(cells * sizeof(double));
   const size_t o_er = take(b->fp32 ? cells * sizeof(float) : 0);
   const size_t o_Ti = take(cells * sizeof(double)), o_Fs = take(cells * b->rsz);
   const size_t o_tal = take((size_t)n_targets * hpic::T_COUNT * sizeof(double));
@@ -460,8 +456,7 @@ int hpic_batch_init(hpic_batch **out, int32_t n_targets, const hpic_target_desc 
   b->pbuf[0] = A + o_p0;
   b->pbuf[1] = A + o_p1;
   b->jall = A + o_j;
-  b->jall_bytes = jv * b->rsz;
-  b->hall = reinterpret_cast<double *>(A + o_H);
+  b->jall_bytes = o_H - o_j + cells * sizeof(double);
   b->items = X + a_items;
   b->d.n = n_targets;
   b->d.wpref = reinterpret_cast<long long *>(X + a_w);

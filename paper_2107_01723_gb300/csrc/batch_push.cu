@@ -44,6 +44,7 @@ static_assert(batch_threads_for(true, 1) == batch_threads_for(true, 2),
 template <typename R>
 __global__ void __launch_bounds__(256) k_batch_plan(const BatchItem<R> *items, BatchDev d) {
   __shared__ long long wt[HPIC_BATCH_MAX_TARGETS], ct[HPIC_BATCH_MAX_TARGETS];
+  after_previous();
   for (int t = threadIdx.x; t < d.n; t += blockDim.x) {
     const BatchItem<R> &it = items[t];
     const long long n = it.cnt->n, st = it.cnt->step;
@@ -98,6 +99,7 @@ k_batch_push(const Consts Krun, const BatchItem<R> *__restrict__ items, BatchDev
   double *tal_s = dyn + kBatchWarps * dep_words<R>() * sizeof(R) / sizeof(double);
   long long *wpref_s = reinterpret_cast<long long *>(tal_s + d.n * kAccN);
   for (int i = threadIdx.x; i < d.n * kAccN; i += blockDim.x) tal_s[i] = 0.0;
+  after_previous();
   for (int t = threadIdx.x; t <= d.n; t += blockDim.x) wpref_s[t] = d.wpref[t];
   __syncthreads();
 
@@ -160,8 +162,9 @@ __device__ __forceinline__ int forward_target(const long long *pref, int t, int 
 
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_batch_inject(const BatchItem<R> *__restrict__ items, BatchDev d, PView<R> p) {
+k_batch_inject(const BatchItem<R> *__restrict__ items, BatchDev d, PView<R> p, bool sorted) {
   extern __shared__ long long ipref_s[];  // n + 1 prefix, then 3 sums per target
+  after_previous();
   double *sum_s = reinterpret_cast<double *>(ipref_s + d.n + 1);
   for (int t = threadIdx.x; t <= d.n; t += blockDim.x) ipref_s[t] = d.ipref[t];
   for (int t = threadIdx.x; t < 3 * d.n; t += blockDim.x) sum_s[t] = 0.0;
@@ -183,7 +186,7 @@ k_batch_inject(const BatchItem<R> *__restrict__ items, BatchDev d, PView<R> p) {
     }
     const BatchItem<R> &it = items[t];
     const long long local = i - ipref_s[t];
-    const long long q = it.cnt->n + local;
+    const long long q = (sorted ? d.snew[t] : it.cnt->n) + local;
     if (q >= it.cap) {
       atomicOr(&it.cnt->flags, 1u);
       continue;
@@ -204,13 +207,15 @@ k_batch_inject(const BatchItem<R> *__restrict__ items, BatchDev d, PView<R> p) {
     if (sum_s[u] != 0.0) atomicAdd(items[u / 3].tv.tal + slot[u % 3], sum_s[u]);
 }
 
-// closes a step of every target: append the injected electrons, advance the clock
+// closes a step of every target: the slots a sort kept, the injected electrons,
+// the clock
 template <typename R>
-__global__ void k_batch_advance(const BatchItem<R> *items, BatchDev d) {
+__global__ void k_batch_advance(const BatchItem<R> *items, BatchDev d, bool sorted) {
+  after_previous();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < d.n; t += gridDim.x * blockDim.x) {
     Counters *cnt = items[t].cnt;
     const long long c = d.ipref[t + 1] - d.ipref[t];
-    const long long n = cnt->n + c, cap = items[t].cap;
+    const long long n = (sorted ? d.snew[t] : cnt->n) + c, cap = items[t].cap;
     cnt->n = n < cap ? n : cap;
     cnt->next_id += c;
     cnt->step += 1;
@@ -226,6 +231,7 @@ template <typename R>
 __global__ void __launch_bounds__(256)
 k_batch_sort_keys(const BatchItem<R> *__restrict__ items, BatchDev d, PView<R> p,
                   uint32_t *keys, uint32_t *ranks, uint32_t *counts, R lead) {
+  after_previous();
   const long long nslot = d.wpref[d.n] * 32;
   int t = 0;
   for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < nslot;
@@ -260,17 +266,12 @@ k_batch_sort_keys(const BatchItem<R> *__restrict__ items, BatchDev d, PView<R> p
 // exclusive offset of its dead bin minus its first offset)
 template <typename R>
 __global__ void k_batch_sort_starts(const BatchItem<R> *items, BatchDev d, const uint32_t *offs) {
+  after_previous();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < d.n; t += gridDim.x * blockDim.x) {
     const long long k0 = d.kpref[t];
     d.sstart[t] = offs[k0];
     d.snew[t] = (long long)offs[k0 + items[t].K.nkeys] - (long long)offs[k0];
   }
-}
-
-template <typename R>
-__global__ void k_batch_sort_finish(const BatchItem<R> *items, BatchDev d) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < d.n; t += gridDim.x * blockDim.x)
-    items[t].cnt->n = d.snew[t];
 }
 
 // ---------------------------------------------------------------- launchers
@@ -331,24 +332,24 @@ void launch_batch_push_ns(const Consts &Krun, const BatchItem<R> *items, BatchDe
                           const SortOut<R> &so) {
   if constexpr (sizeof(R) == 8) {  // FP64: one or two blocks per SM
     if (blocks_per_sm <= 1)
-      k_batch_push<R, 1, NS, SORT><<<grid, batch_threads<R, 1>(), sm, st>>>(Krun, items, d, p,
-                                                                            table, so);
+      launch_chained(k_batch_push<R, 1, NS, SORT>, grid, batch_threads<R, 1>(), sm, st, Krun, items, d,
+                     p, table, so);
     else
-      k_batch_push<R, 2, NS, SORT><<<grid, batch_threads<R, 2>(), sm, st>>>(Krun, items, d, p,
-                                                                            table, so);
+      launch_chained(k_batch_push<R, 2, NS, SORT>, grid, batch_threads<R, 2>(), sm, st, Krun, items, d,
+                     p, table, so);
   } else {  // FP32: two to five (one runs the two-block code)
     if (blocks_per_sm <= 2)
-      k_batch_push<R, 2, NS, SORT><<<grid, batch_threads<R, 2>(), sm, st>>>(Krun, items, d, p,
-                                                                            table, so);
+      launch_chained(k_batch_push<R, 2, NS, SORT>, grid, batch_threads<R, 2>(), sm, st, Krun, items, d,
+                     p, table, so);
     else if (blocks_per_sm == 3)
-      k_batch_push<R, 3, NS, SORT><<<grid, batch_threads<R, 3>(), sm, st>>>(Krun, items, d, p,
-                                                                            table, so);
+      launch_chained(k_batch_push<R, 3, NS, SORT>, grid, batch_threads<R, 3>(), sm, st, Krun, items, d,
+                     p, table, so);
     else if (blocks_per_sm == 4)
-      k_batch_push<R, 4, NS, SORT><<<grid, batch_threads<R, 4>(), sm, st>>>(Krun, items, d, p,
-                                                                            table, so);
+      launch_chained(k_batch_push<R, 4, NS, SORT>, grid, batch_threads<R, 4>(), sm, st, Krun, items, d,
+                     p, table, so);
     else
-      k_batch_push<R, 5, NS, SORT><<<grid, batch_threads<R, 5>(), sm, st>>>(Krun, items, d, p,
-                                                                            table, so);
+      launch_chained(k_batch_push<R, 5, NS, SORT>, grid, batch_threads<R, 5>(), sm, st, Krun, items, d,
+                     p, table, so);
   }
 }
 
@@ -373,15 +374,15 @@ void launch_batch_push(const Consts &Krun, const BatchItem<R> *items, BatchDev d
 }
 
 template <typename R>
-void launch_batch_inject(const BatchItem<R> *items, BatchDev d, PView<R> p, int grid,
+void launch_batch_inject(const BatchItem<R> *items, BatchDev d, PView<R> p, bool sorted, int grid,
                          cudaStream_t st) {
   const size_t sm = (d.n + 1) * sizeof(long long) + 3 * d.n * sizeof(double);
-  k_batch_inject<R><<<grid, 256, sm, st>>>(items, d, p);
+  launch_chained(k_batch_inject<R>, grid, 256, sm, st, items, d, p, sorted);
 }
 
 template <typename R>
-void launch_batch_advance(const BatchItem<R> *items, BatchDev d, cudaStream_t st) {
-  k_batch_advance<R><<<1, 256, 0, st>>>(items, d);
+void launch_batch_advance(const BatchItem<R> *items, BatchDev d, bool sorted, cudaStream_t st) {
+  launch_chained(k_batch_advance<R>, 1, 256, 0, st, items, d, sorted);
 }
 
 template <typename R>
@@ -390,15 +391,9 @@ int launch_batch_sort_keys(const BatchItem<R> *items, BatchDev d, PView<R> p, ui
                            long long nkeys_total, int grid, cudaStream_t st, double lead) {
   cudaMemsetAsync(counts, 0, nkeys_total * sizeof(uint32_t), st);
   k_batch_sort_keys<R><<<grid, 256, 0, st>>>(items, d, p, keys, ranks, counts, R(lead));
-  const int launches = 1 + launch_scan(counts, nkeys_total, partials, st);
-  k_batch_sort_starts<R><<<1, 256, 0, st>>>(items, d, counts);
+  const int launches = 1 + launch_scan(counts, nkeys_total, partials, st, true);
+  launch_chained(k_batch_sort_starts<R>, 1, 256, 0, st, items, d, counts);
   return launches + 1;
-}
-
-template <typename R>
-int launch_batch_sort_finish(const BatchItem<R> *items, BatchDev d, cudaStream_t st) {
-  k_batch_sort_finish<R><<<1, 256, 0, st>>>(items, d);
-  return 1;
 }
 
 #define HPIC_INST(R)                                                                            \
@@ -406,13 +401,12 @@ int launch_batch_sort_finish(const BatchItem<R> *items, BatchDev d, cudaStream_t
   template void launch_batch_push<R>(const Consts &, const BatchItem<R> *, BatchDev, PView<R>,  \
                                      const R *, int, int, bool, cudaStream_t,                   \
                                      const SortOut<R> &);                                       \
-  template void launch_batch_inject<R>(const BatchItem<R> *, BatchDev, PView<R>, int,           \
+  template void launch_batch_inject<R>(const BatchItem<R> *, BatchDev, PView<R>, bool, int,     \
                                        cudaStream_t);                                           \
-  template void launch_batch_advance<R>(const BatchItem<R> *, BatchDev, cudaStream_t);          \
+  template void launch_batch_advance<R>(const BatchItem<R> *, BatchDev, bool, cudaStream_t);    \
   template int launch_batch_sort_keys<R>(const BatchItem<R> *, BatchDev, PView<R>, uint32_t *, \
                                          uint32_t *, uint32_t *, uint32_t *, long long, int,    \
-                                         cudaStream_t, double);                                 \
-  template int launch_batch_sort_finish<R>(const BatchItem<R> *, BatchDev, cudaStream_t);
+                                         cudaStream_t, double);
 HPIC_INST(float)
 HPIC_INST(double)
 #undef HPIC_INST

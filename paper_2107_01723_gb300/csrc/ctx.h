@@ -42,7 +42,7 @@ struct hpic_ctx {
   size_t xfer_bytes = 0;
   // grid
   void *fields = nullptr;  // E[3], B[3] of R, each nvec long, vstride apart
-  void *jfield = nullptr;  // J[3], vstride apart (just after B in a single context)
+  void *jfield = nullptr;  // J[3], vstride apart (just after B in a single context), then H
   long long vstride = 0;   // nvec + >= 4 padding, a multiple of 64 (aligned vector access)
   double *T = nullptr, *eta = nullptr, *H = nullptr;
   void *eta_r = nullptr;  // FP32 copy of eta read by the FP32 field solve (mixed precision)

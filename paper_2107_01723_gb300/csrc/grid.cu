@@ -14,16 +14,20 @@ namespace hpic {
 
 template <typename R>
 __global__ void __launch_bounds__(256, kFieldBlocksPerSm) k_efield(const FieldK<R> K, GView<R> g) {
+  after_previous();
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < K.nvec; q += gridDim.x * blockDim.x)
     efield_node(K, g, q);
 }
 
 template <typename R>
 __global__ void __launch_bounds__(256, kFieldBlocksPerSm)
-k_bheat(const FieldK<R> K, GView<R> g, TallyView tv) {
+k_bheat(const FieldK<R> K, GView<R> g, TallyView tv, const StepEnd end) {
   __shared__ double sum;
   if (threadIdx.x == 0) sum = 0.0;
   __syncthreads();
+  after_previous();
+  // nothing in this kernel or after it in the step reads the counters
+  if (end.cnt && blockIdx.x == 0 && threadIdx.x == 0) close_step(end);
   WideSum<R> ohm;
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < K.nvec; q += gridDim.x * blockDim.x)
     bheat_node(K, g, q, ohm);
@@ -68,6 +72,7 @@ __global__ void __launch_bounds__(256, kBatchFieldBlocksPerSm)
 k_batch_efield(const BatchItem<R> *items, BatchDev d) {
   extern __shared__ long long npref_s[];
   __shared__ FieldHot<R> hot[8];
+  after_previous();
   for (int t = threadIdx.x; t <= d.n; t += blockDim.x) npref_s[t] = d.npref[t];
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -88,6 +93,7 @@ k_batch_bheat(const BatchItem<R> *items, BatchDev d) {
   extern __shared__ long long npref_s[];
   __shared__ FieldHot<R> hot[8];
   double *ohm_s = reinterpret_cast<double *>(npref_s + d.n + 1);
+  after_previous();
   for (int t = threadIdx.x; t <= d.n; t += blockDim.x) npref_s[t] = d.npref[t];
   for (int t = threadIdx.x; t < d.n; t += blockDim.x) ohm_s[t] = 0.0;
   __syncthreads();
@@ -119,6 +125,7 @@ template <typename R>
 __global__ void __launch_bounds__(256)
 k_sort_keys(const Consts K, PView<R> p, const Counters *cnt, uint32_t *keys, uint32_t *counts,
             R lead, uint32_t *ranks) {
+  after_previous();
   const long long n = cnt->n;
   for (long long ip = blockIdx.x * (long long)blockDim.x + threadIdx.x; ip < n;
        ip += (long long)gridDim.x * blockDim.x) {
@@ -151,6 +158,7 @@ k_sort_keys(const Consts K, PView<R> p, const Counters *cnt, uint32_t *keys, uin
 __global__ void __launch_bounds__(1024) k_scan_tiles(const uint32_t *counts, long long m,
                                                      uint32_t *partials) {
   __shared__ uint32_t ws[32];
+  after_previous();
   const long long base = (long long)blockIdx.x * kScanTile;
   uint32_t s = 0;
   for (int t = threadIdx.x; t < kScanTile; t += blockDim.x) {
@@ -173,6 +181,7 @@ __global__ void __launch_bounds__(1024) k_scan_top(uint32_t *partials, int ntile
   __shared__ uint32_t carry;
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
+  after_previous();
   for (int base = 0; base < ntiles; base += blockDim.x) {
     const int t = base + threadIdx.x;
     const uint32_t v = t < ntiles ? partials[t] : 0u;
@@ -211,6 +220,7 @@ __global__ void __launch_bounds__(1024) k_scan_apply(uint32_t *counts, long long
   __shared__ uint32_t ws[32];
   __shared__ uint32_t carry;
   const long long base = (long long)blockIdx.x * kScanTile;
+  after_previous();
   if (threadIdx.x == 0) carry = partials[blockIdx.x];
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -240,6 +250,65 @@ __global__ void __launch_bounds__(1024) k_scan_apply(uint32_t *counts, long long
     __syncthreads();
     if (threadIdx.x == blockDim.x - 1) carry = incl;
     __syncthreads();
+  }
+}
+
+// The same of a short range (up to kScanShort) by one block: a thread takes
+// `per` consecutive counts, all loaded before the block's one scan.
+constexpr int kScanPer = 16;  // counts per thread at most, a multiple of 4
+constexpr long long kScanShort = 1024 * kScanPer;
+
+__global__ void __launch_bounds__(1024) k_scan_short(uint32_t *counts, int m) {
+  __shared__ uint32_t ws[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = ((m + 1023) / 1024 + 3) & ~3, first = (int)threadIdx.x * per;
+  after_previous();
+  uint4 v[kScanPer / 4];
+  uint32_t s = 0;
+#pragma unroll
+  for (int q = 0; q < kScanPer / 4; ++q) {
+    const int at = first + 4 * q;
+    v[q] = make_uint4(0u, 0u, 0u, 0u);
+    if (4 * q < per) {
+      if (at + 3 < m) {
+        v[q] = *reinterpret_cast<const uint4 *>(counts + at);
+      } else {
+        if (at < m) v[q].x = counts[at];
+        if (at + 1 < m) v[q].y = counts[at + 1];
+        if (at + 2 < m) v[q].z = counts[at + 2];
+      }
+    }
+    s += v[q].x + v[q].y + v[q].z + v[q].w;
+  }
+  uint32_t x = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) ws[warp] = x;
+  __syncthreads();
+  uint32_t z = ws[lane];  // every warp scans the warps' sums for itself
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, z, o);
+    if (lane >= o) z += y;
+  }
+  const uint32_t before = __shfl_sync(0xffffffffu, z, warp ? warp - 1 : 0);
+  uint32_t run = (warp ? before : 0u) + x - s;
+#pragma unroll
+  for (int q = 0; q < kScanPer / 4; ++q) {
+    const int at = first + 4 * q;
+    if (4 * q >= per) break;
+    const uint4 o = make_uint4(run, run + v[q].x, run + v[q].x + v[q].y, run + v[q].x + v[q].y + v[q].z);
+    run = o.w + v[q].w;
+    if (at + 3 < m) {
+      *reinterpret_cast<uint4 *>(counts + at) = o;
+    } else {
+      if (at < m) counts[at] = o.x;
+      if (at + 1 < m) counts[at + 1] = o.y;
+      if (at + 2 < m) counts[at + 2] = o.z;
+    }
   }
 }
 
@@ -349,19 +418,29 @@ __global__ void __launch_bounds__(256) k_field_energy(const Consts K, GView<R> g
 // ---------------------------------------------------------------- launchers
 template <typename R>
 void launch_efield(const Consts &K, GView<R> g, int grid, cudaStream_t st) {
-  k_efield<R><<<grid, 256, 0, st>>>(make_field<R>(K), g);
+  launch_chained(k_efield<R>, grid, 256, 0, st, make_field<R>(K), g);
 }
 
 template <typename R>
-void launch_bheat(const Consts &K, GView<R> g, TallyView tv, int grid, cudaStream_t st) {
-  k_bheat<R><<<grid, 256, 0, st>>>(make_field<R>(K), g, tv);
+void launch_bheat(const Consts &K, GView<R> g, TallyView tv, const StepEnd &end, int grid,
+                  cudaStream_t st) {
+  launch_chained(k_bheat<R>, grid, 256, 0, st, make_field<R>(K), g, tv, end);
 }
 
-int launch_scan(uint32_t *counts, long long m, uint32_t *partials, cudaStream_t st) {
+// Up to kScanShort counts one block scans: one launch for three.  (8e3 counts
+// of five small targets: 3.1 us, for three kernels of 7.4 us and their gaps;
+// 32769 counts of 32^3 cells in 36 per thread: 8.3 us, no gain.)
+int launch_scan(uint32_t *counts, long long m, uint32_t *partials, cudaStream_t st, bool chained) {
+  if (m <= kScanShort) {
+    if (chained) launch_chained(k_scan_short, 1, 1024, 0, st, counts, (int)m);
+    else k_scan_short<<<1, 1024, 0, st>>>(counts, (int)m);
+    return 1;
+  }
   const int ntiles = (int)((m + kScanTile - 1) / kScanTile);
-  k_scan_tiles<<<ntiles, 1024, 0, st>>>(counts, m, partials);
-  k_scan_top<<<1, 1024, 0, st>>>(partials, ntiles);
-  k_scan_apply<<<ntiles, 1024, 0, st>>>(counts, m, partials);
+  if (chained) launch_chained(k_scan_tiles, ntiles, 1024, 0, st, counts, m, partials);
+  else k_scan_tiles<<<ntiles, 1024, 0, st>>>(counts, m, partials);
+  launch_chained(k_scan_top, 1, 1024, 0, st, partials, ntiles);
+  launch_chained(k_scan_apply, ntiles, 1024, 0, st, counts, m, partials);
   return 3;
 }
 
@@ -371,10 +450,10 @@ int launch_sort(const Consts &K, PView<R> src, PView<R> dst, Counters *cnt, uint
   const long long m = K.nkeys + 1;
   cudaMemsetAsync(counts, 0, m * sizeof(uint32_t), st);
   k_sort_keys<R><<<grid, 256, 0, st>>>(K, src, cnt, keys, counts, R(lead * K.cdt_dx), nullptr);
-  launch_scan(counts, m, partials, st);
+  const int launches = launch_scan(counts, m, partials, st);
   k_sort_scatter<R><<<grid, 256, 0, st>>>(K, src, dst, cnt, keys, counts);
   k_sort_finish<<<1, 32, 0, st>>>(cnt, counts, K.nkeys);
-  return 6;
+  return 3 + launches;
 }
 
 template <typename R>
@@ -383,12 +462,7 @@ int launch_sort_keys(const Consts &K, PView<R> p, Counters *cnt, uint32_t *keys,
   const long long m = K.nkeys + 1;
   cudaMemsetAsync(counts, 0, m * sizeof(uint32_t), st);
   k_sort_keys<R><<<grid, 256, 0, st>>>(K, p, cnt, keys, counts, R(lead * K.cdt_dx), ranks);
-  return 1 + launch_scan(counts, m, partials, st);
-}
-
-int launch_sort_finish(const Consts &K, Counters *cnt, const uint32_t *offsets, cudaStream_t st) {
-  k_sort_finish<<<1, 32, 0, st>>>(cnt, offsets, K.nkeys);
-  return 1;
+  return 1 + launch_scan(counts, m, partials, st, true);
 }
 
 void launch_table(const Consts &K, double k_min, double E_max, double *t64, float *t32,
@@ -400,13 +474,13 @@ void launch_table(const Consts &K, double k_min, double E_max, double *t64, floa
 
 template <typename R>
 void launch_batch_efield(const BatchItem<R> *items, BatchDev d, int grid, cudaStream_t st) {
-  k_batch_efield<R><<<grid, 256, (d.n + 1) * sizeof(long long), st>>>(items, d);
+  launch_chained(k_batch_efield<R>, grid, 256, (d.n + 1) * sizeof(long long), st, items, d);
 }
 
 template <typename R>
 void launch_batch_bheat(const BatchItem<R> *items, BatchDev d, int grid, cudaStream_t st) {
   const size_t sm = (d.n + 1) * sizeof(long long) + d.n * sizeof(double);
-  k_batch_bheat<R><<<grid, 256, sm, st>>>(items, d);
+  launch_chained(k_batch_bheat<R>, grid, 256, sm, st, items, d);
 }
 
 template <typename R>
@@ -596,7 +670,8 @@ void launch_scale_out(const T *src, long long n, double scale, double *out, int 
 
 #define HPIC_INST(R)                                                                          \
   template void launch_efield<R>(const Consts &, GView<R>, int, cudaStream_t);                \
-  template void launch_bheat<R>(const Consts &, GView<R>, TallyView, int, cudaStream_t);      \
+  template void launch_bheat<R>(const Consts &, GView<R>, TallyView, const StepEnd &, int,    \
+                                cudaStream_t);                                                \
   template int launch_sort<R>(const Consts &, PView<R>, PView<R>, Counters *, uint32_t *,     \
                               uint32_t *, uint32_t *, int, cudaStream_t, double);             \
   template int launch_sort_keys<R>(const Consts &, PView<R>, Counters *, uint32_t *, uint32_t *, \

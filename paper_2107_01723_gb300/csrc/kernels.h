@@ -3,12 +3,44 @@
 
 #include <cuda_runtime.h>
 
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
 #include "hpic.h"
 
 namespace hpic {
+
+// Kernels of a step follow one another in a stream.  A chained launch lets the
+// next one's blocks take their places while the last one's are finishing
+// (programmatic dependent launch) instead of after its end has been reported;
+// every kernel of the chain begins with after_previous(), which waits for the
+// kernels before it to end and their stores to be visible, so only the launch
+// itself overlaps.  No kernel releases the next one early: its blocks would
+// take the SMs that happen to be free first and crowd there (FP64, 1e5
+// electrons: a step 226 instead of 198 us).  Small runs are made of such gaps:
+// with one clearing for two, the step closed by the heating kernel and chained
+// launches, a step of 1e5 electrons (FP32) went from 50 to 37 us, of 2e3
+// electrons from 33 to 25 us.  Only a launch that directly follows another
+// kernel of the same call is chained.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), int grid, int threads, size_t smem,
+                           cudaStream_t st, A &&...args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // particle storage: structure of arrays, positions in cells, momenta u = p/(m_e c)
 template <typename R>
@@ -253,10 +285,27 @@ template <typename R>
 void launch_push(const Consts &K, PView<R> p, GView<R> g, const R *table, Counters *cnt,
                  TallyView tv, long long cap, int sm_count, cudaStream_t st,
                  const SortOut<R> &so, const KeyOut<R> &ko);
+// What closes a step: the slots kept by a sort (kept: their count on the
+// device, or NULL), the injected electrons and the clock.  The heating kernel
+// does it where nothing comes after it, else launch_advance.
+struct StepEnd {
+  Counters *cnt;  // NULL: not here
+  const uint32_t *kept;
+  long long cap;
+};
+__device__ __forceinline__ void close_step(const StepEnd &end) {
+  Counters *cnt = end.cnt;
+  const long long c = cnt->inj_cnt;
+  const long long n = (end.kept ? (long long)*end.kept : cnt->n) + c;
+  cnt->n = n < end.cap ? n : end.cap;
+  cnt->next_id += c;
+  cnt->step += 1;
+  cnt->inj_cnt = 0;
+}
 template <typename R>
-void launch_inject(const Consts &K, PView<R> p, Counters *cnt, long long cap, TallyView tv,
-                   int grid, cudaStream_t st);
-void launch_advance(Counters *cnt, long long cap, cudaStream_t st);
+void launch_inject(const Consts &K, PView<R> p, const StepEnd &end, TallyView tv, int grid,
+                   cudaStream_t st);
+void launch_advance(const StepEnd &end, cudaStream_t st);
 // bulk seeding (two launches); mean kinetic energy in m_e c^2
 template <typename R>
 void launch_seed(const Consts &K, PView<R> p, Counters *cnt, long long cap, long long count,
@@ -265,7 +314,8 @@ void launch_seed(const Consts &K, PView<R> p, Counters *cnt, long long cap, long
 template <typename R>
 void launch_efield(const Consts &K, GView<R> g, int grid, cudaStream_t st);
 template <typename R>
-void launch_bheat(const Consts &K, GView<R> g, TallyView tv, int grid, cudaStream_t st);
+void launch_bheat(const Consts &K, GView<R> g, TallyView tv, const StepEnd &end, int grid,
+                  cudaStream_t st);
 
 // counting sort by cell: keys/counts/offsets are scratch; electrons are keyed
 // by the cell they reach `lead` steps ahead at their current velocity (0: the
@@ -283,12 +333,11 @@ inline double sort_lead(int interval) { return interval > 0 ? 0.5 * (interval + 
 // The counting sort folded into a step: keys, ranks (each slot's place among
 // the slots of its key) and the scanned offsets of the electrons in p, keyed
 // `lead` steps ahead; the step's push then writes each electron to its
-// sorted slot (SortOut) and launch_sort_finish sets the slot count to the
-// electrons kept.  Return launches made.
+// sorted slot (SortOut) and the end of the step sets the slot count to the
+// electrons kept (StepEnd).  Return launches made.
 template <typename R>
 int launch_sort_keys(const Consts &K, PView<R> p, Counters *cnt, uint32_t *keys, uint32_t *ranks,
                      uint32_t *counts, uint32_t *partials, int grid, cudaStream_t st, double lead);
-int launch_sort_finish(const Consts &K, Counters *cnt, const uint32_t *offsets, cudaStream_t st);
 
 void launch_table(const Consts &K, double k_min, double E_max, double *t64, float *t32,
                   cudaStream_t st);
@@ -335,10 +384,10 @@ void launch_batch_push(const Consts &Krun, const BatchItem<R> *items, BatchDev d
                        const R *table, int sm_count, int blocks_per_sm, bool single,
                        cudaStream_t st, const SortOut<R> &so);
 template <typename R>
-void launch_batch_inject(const BatchItem<R> *items, BatchDev d, PView<R> p, int grid,
+void launch_batch_inject(const BatchItem<R> *items, BatchDev d, PView<R> p, bool sorted, int grid,
                          cudaStream_t st);
 template <typename R>
-void launch_batch_advance(const BatchItem<R> *items, BatchDev d, cudaStream_t st);
+void launch_batch_advance(const BatchItem<R> *items, BatchDev d, bool sorted, cudaStream_t st);
 template <typename R>
 void launch_batch_efield(const BatchItem<R> *items, BatchDev d, int grid, cudaStream_t st);
 template <typename R>
@@ -352,14 +401,14 @@ template <typename R>
 int launch_batch_sort_keys(const BatchItem<R> *items, BatchDev d, PView<R> p, uint32_t *keys,
                            uint32_t *ranks, uint32_t *counts, uint32_t *partials,
                            long long nkeys_total, int grid, cudaStream_t st, double lead);
-template <typename R>
-int launch_batch_sort_finish(const BatchItem<R> *items, BatchDev d, cudaStream_t st);
 // counts summed per block of the scan; the partials scratch of a scan of m
 // counts holds scan_partials(m) words
 constexpr long long kScanTile = 4096;
 constexpr long long scan_partials(long long m) { return (m + kScanTile - 1) / kScanTile + 1; }
 // exclusive scan of counts[0, m) in place (partials: scratch of
-// scan_partials(m) words); returns launches made
-int launch_scan(uint32_t *counts, long long m, uint32_t *partials, cudaStream_t st);
+// scan_partials(m) words); chained: it follows a kernel of the same call;
+// returns launches made
+int launch_scan(uint32_t *counts, long long m, uint32_t *partials, cudaStream_t st,
+                bool chained = false);
 
 }  // namespace hpic

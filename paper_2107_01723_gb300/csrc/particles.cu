@@ -36,6 +36,7 @@ template <typename R, int NS, int MODE>
 __global__ void __launch_bounds__(push_threads<R>(MODE), push_blocks_per_sm<R>(MODE))
 k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__restrict__ tab,
        Counters *cnt, TallyView tv, const SortOut<R> so, const KeyOut<R> ko) {
+  after_previous();
   const long long n = cnt->n;
   if (blockIdx.x * (long long)blockDim.x >= n) return;  // the whole block: no slot for it
   __shared__ double sums[kAccN];  // the tally sums of the block
@@ -83,13 +84,14 @@ k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__rest
 // while g(t) >= g_min, each of weight inj_unit sqrt(f g) and local mean
 // energy a0 sqrt(f g) m_e c^2; ids run cell by cell in the cells' order.
 template <typename R>
-__device__ void inject_gauss(const Consts &K, PView<R> p, Counters *cnt, long long cap,
-                             TallyView tv, double *smem) {
-  const long long st = cnt->step;
+__device__ void inject_gauss(const Consts &K, PView<R> p, const StepEnd &end, TallyView tv,
+                             double *smem) {
+  Counters *cnt = end.cnt;
+  const long long st = cnt->step, cap = end.cap;
   const double tm = (double)st + 0.5 - K.t_pk;
   const double g = exp(-K.g_c * tm * tm);
   const long long c = g >= K.g_min ? K.per_cell * K.n_inj_cells : 0;
-  const long long n0 = cnt->n, id0 = cnt->next_id;
+  const long long n0 = end.kept ? (long long)*end.kept : cnt->n, id0 = cnt->next_id;
   const uint32_t step = (uint32_t)st;
   const double sg = sqrt(g);
   const InjCell *cells = static_cast<const InjCell *>(K.inj_cells);
@@ -118,17 +120,19 @@ __device__ void inject_gauss(const Consts &K, PView<R> p, Counters *cnt, long lo
 
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_inject(const Consts K, PView<R> p, Counters *cnt, long long cap, TallyView tv) {
+k_inject(const Consts K, PView<R> p, const StepEnd end, TallyView tv) {
   __shared__ double smem[3 * 32];
+  after_previous();
   if (K.weighted) {
-    inject_gauss(K, p, cnt, cap, tv, smem);
+    inject_gauss(K, p, end, tv, smem);
     return;
   }
-  const long long st = cnt->step;
+  Counters *cnt = end.cnt;
+  const long long st = cnt->step, cap = end.cap;
   if (st >= K.n_inj_steps) return;
   const long long S = K.n_inj_steps, N = K.n_macro;
   const long long c = (N * (st + 1)) / S - (N * st) / S;
-  const long long n0 = cnt->n, id0 = cnt->next_id;
+  const long long n0 = end.kept ? (long long)*end.kept : cnt->n, id0 = cnt->next_id;
   const uint32_t step = (uint32_t)st;
   double e_inj = 0.0, n_inj = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < c;
@@ -211,16 +215,9 @@ template void launch_seed<float>(const Consts &, PView<float>, Counters *, long 
 template void launch_seed<double>(const Consts &, PView<double>, Counters *, long long,
                                   long long, double, TallyView, int, cudaStream_t);
 
-// closes a step: append the injected electrons, advance the clock
-__global__ void k_advance(Counters *cnt, long long cap) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const long long c = cnt->inj_cnt;
-    long long n = cnt->n + c;
-    cnt->n = n < cap ? n : cap;
-    cnt->next_id += c;
-    cnt->step += 1;
-    cnt->inj_cnt = 0;
-  }
+__global__ void k_advance(const StepEnd end) {
+  after_previous();
+  if (blockIdx.x == 0 && threadIdx.x == 0) close_step(end);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -259,8 +256,12 @@ void launch_push_mode(const Consts &K, const HotK<R> &h, PView<R> p, GView<R> g,
   constexpr int threads = push_threads<R>(MODE);
   const long long want = (cap + threads - 1) / threads;
   const long long wave = (long long)sm_count * push_blocks_per_sm<R>(MODE);
-  k_push<R, NS, MODE><<<(int)(want < wave ? want : wave), threads, push_stage_bytes<R, MODE>(), st>>>(
-      K, h, p, g, table, cnt, tv, so, ko);
+  const int grid = (int)(want < wave ? want : wave);
+  constexpr size_t smem = push_stage_bytes<R, MODE>();
+  if (MODE == kPushSort)  // it follows the sort's scan
+    launch_chained(k_push<R, NS, MODE>, grid, threads, smem, st, K, h, p, g, table, cnt, tv, so, ko);
+  else
+    k_push<R, NS, MODE><<<grid, threads, smem, st>>>(K, h, p, g, table, cnt, tv, so, ko);
 }
 
 template <typename R, int NS>
@@ -293,13 +294,13 @@ void launch_push(const Consts &K, PView<R> p, GView<R> g, const R *table, Counte
 }
 
 template <typename R>
-void launch_inject(const Consts &K, PView<R> p, Counters *cnt, long long cap, TallyView tv,
-                   int grid, cudaStream_t st) {
-  k_inject<R><<<grid, 256, 0, st>>>(K, p, cnt, cap, tv);
+void launch_inject(const Consts &K, PView<R> p, const StepEnd &end, TallyView tv, int grid,
+                   cudaStream_t st) {
+  launch_chained(k_inject<R>, grid, 256, 0, st, K, p, end, tv);
 }
 
-void launch_advance(Counters *cnt, long long cap, cudaStream_t st) {
-  k_advance<<<1, 32, 0, st>>>(cnt, cap);
+void launch_advance(const StepEnd &end, cudaStream_t st) {
+  launch_chained(k_advance, 1, 32, 0, st, end);
 }
 
 template void launch_push<float>(const Consts &, PView<float>, GView<float>, const float *,
@@ -308,9 +309,9 @@ template void launch_push<float>(const Consts &, PView<float>, GView<float>, con
 template void launch_push<double>(const Consts &, PView<double>, GView<double>, const double *,
                                   Counters *, TallyView, long long, int, cudaStream_t,
                                   const SortOut<double> &, const KeyOut<double> &);
-template void launch_inject<float>(const Consts &, PView<float>, Counters *, long long, TallyView,
-                                   int, cudaStream_t);
-template void launch_inject<double>(const Consts &, PView<double>, Counters *, long long,
-                                    TallyView, int, cudaStream_t);
+template void launch_inject<float>(const Consts &, PView<float>, const StepEnd &, TallyView, int,
+                                   cudaStream_t);
+template void launch_inject<double>(const Consts &, PView<double>, const StepEnd &, TallyView, int,
+                                    cudaStream_t);
 
 }  // namespace hpic
