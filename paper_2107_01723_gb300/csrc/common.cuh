@@ -122,8 +122,15 @@ __device__ __forceinline__ U4 philox10(uint32_t c0, uint32_t c1, uint32_t c2, ui
 
 // open-interval uniform from the top 23 bits; exact in float and double
 template <typename R>
-__device__ __forceinline__ R unif(uint32_t x) {
-  return (R(x >> 9) + R(0.5)) * R(1.0 / 8388608.0);
+__device__ __forceinline__ R unif(uint32_t x);
+template <>
+__device__ __forceinline__ float unif<float>(uint32_t x) {
+  return ((float)(x >> 9) + 0.5f) * (1.0f / 8388608.0f);
+}
+template <>
+__device__ __forceinline__ double unif<double>(uint32_t x) {  // 1 + m 2^-23 by its bits
+  const uint32_t m = x >> 9;
+  return __hiloint2double((int)(0x3ff00000u | (m >> 3)), (int)(m << 29)) - (1.0 - 1.0 / 16777216.0);
 }
 
 // ---------------------------------------------------------------- math wrappers
@@ -236,6 +243,103 @@ __device__ __forceinline__ float m_div_near(float n, float d) {
   return fmaf(fmaf(-q, d, n), y, q);
 }
 __device__ __forceinline__ double m_div_near(double n, double d) { return n * m_rcp(d); }
+// p = sqrt(x) near-rounded, and 1/p
+__device__ __forceinline__ void m_sqrt_both(float x, float &p, float &inv) {
+  inv = rsqrtf(x);
+  const float s = x * inv;
+  p = fmaf(fmaf(-s, s, x), 0.5f * inv, s);
+}
+__device__ __forceinline__ void m_sqrt_both(double x, double &p, double &inv) {
+  inv = m_rsqrt(x);
+  p = x * inv;
+}
+
+// ---- tables of the FP64 push
+// Logarithms and the circle's functions cost 20 to 30 FP64 operations each in
+// full generality.  By Tang's table-driven methods (ACM TOMS 15(2), 1989, and
+// 16(4), 1990) the logarithm of a normal number takes ten, and sine and cosine
+// of a 23-bit deviate of the circle, whose sector and rest are exact integers,
+// thirteen.  All errors are of a few 1e-16 of 1.  With them, small-angle series
+// and deviates and range tests by the bits the FP64 push of 1e6 electrons went
+// from 1290 to 1062 us.
+struct Fp64Tables {
+  double c[256], l[256];    // c: a 24-bit reciprocal of 1 + (j + 1/2)/256; l = -ln c
+  double cs[256], sn[256];  // of the angle 2 pi (j + 1/2)/256
+  static constexpr double ln(double x) {  // x in [1/2, 1]
+    const double y = (x - 1.0) / (x + 1.0), y2 = y * y;
+    double s = 0.0;
+    for (int k = 41; k >= 1; k -= 2) s = s * y2 + 1.0 / k;
+    return 2.0 * y * s;
+  }
+  static constexpr double sine(double a) {  // |a| <= pi/4
+    double s = 0.0;
+    for (int k = 19; k >= 1; k -= 2) s = 1.0 - s * a * a / ((k + 1) * (k + 2));
+    return a * s;
+  }
+  static constexpr double cosine(double a) {
+    double s = 0.0;
+    for (int k = 20; k >= 0; k -= 2) s = 1.0 - s * a * a / ((k + 1) * (k + 2));
+    return s;
+  }
+  constexpr Fp64Tables() : c(), l(), cs(), sn() {
+    constexpr double pi = 3.14159265358979323846;
+    for (int j = 0; j < 256; ++j) {
+      c[j] = (double)(float)(512.0 / (512.0 + 2 * j + 1));
+      l[j] = -ln(c[j]);
+      const int q = j / 64, r = j % 64;  // quadrant, and 2 r + 1 512ths of the circle in it
+      const bool far = r >= 32;          // beyond pi/4: by the complement
+      const double a = (far ? 127 - 2 * r : 2 * r + 1) * pi / 256.0;
+      const double s = far ? cosine(a) : sine(a), o = far ? sine(a) : cosine(a);
+      cs[j] = q == 0 ? o : (q == 1 ? -s : (q == 2 ? -o : s));
+      sn[j] = q == 0 ? s : (q == 1 ? o : (q == 2 ? -s : -o));
+    }
+  }
+};
+static __device__ const Fp64Tables kFp64 = Fp64Tables();
+
+__device__ __forceinline__ double table_log(double x) {
+  const int hi = __double2hiint(x);
+  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // not positive and normal
+  const int j = (hi >> 12) & 255;
+  const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
+  const double k = __hiloint2double(0x43300000, ((hi >> 20) - 1023) ^ (int)0x80000000) -
+                   4503601774854144.0;  // by the bits of k + 2^52 + 2^31
+  const double r = fma(m, __ldg(kFp64.c + j), -1.0);  // |r| < 2^-9 + 2^-23
+  double q = fma(r, -1.0 / 6.0, 0.2);
+  q = fma(r, q, -0.25);
+  q = fma(r, q, 1.0 / 3.0);
+  q = fma(r, q, -0.5);
+  q = fma(r, q, 1.0);
+  return fma(r, q, fma(k, 0.693147180559945309417232, __ldg(kFp64.l + j)));
+}
+// cos (and sin) of 2 pi u, u = (m + 1/2) 2^-23 the deviate of x
+__device__ __forceinline__ void table_turn(uint32_t x, double &s, double &c) {
+  const uint32_t m = x >> 9;
+  const int j = (int)(m >> 15), f = 2 * (int)(m & 0x7fffu) - 32767;  // 2^-24ths from the middle
+  const double a = (double)f * (3.14159265358979323846 / 8388608.0), t = a * a;
+  const double sa = fma(a * t, fma(t, 1.0 / 120.0, -1.0 / 6.0), a);
+  const double ca = fma(t, fma(t, fma(t, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
+  const double cj = __ldg(kFp64.cs + j), sj = __ldg(kFp64.sn + j);
+  c = fma(cj, ca, -(sj * sa));
+  s = fma(sj, ca, cj * sa);
+}
+
+// the push's logarithms: of a deviate, and the quick one
+__device__ __forceinline__ float p_log(float x) { return logf(x); }
+__device__ __forceinline__ double p_log(double x) { return table_log(x); }
+__device__ __forceinline__ float p_flog(float x) { return __logf(x); }
+__device__ __forceinline__ double p_flog(double x) { return table_log(x); }
+// sine and cosine of the deviate x of the circle; its cosine for a normal deviate
+__device__ __forceinline__ void p_turn(uint32_t x, float &s, float &c) {
+  m_sincos2pi(unif<float>(x), &s, &c);
+}
+__device__ __forceinline__ void p_turn(uint32_t x, double &s, double &c) { table_turn(x, s, c); }
+__device__ __forceinline__ void p_cos_turn(uint32_t x, float &c) { c = m_fcos2pi(unif<float>(x)); }
+__device__ __forceinline__ void p_cos_turn(uint32_t x, double &c) {
+  double s;
+  table_turn(x, s, c);
+}
+
 // sine and cosine of a deflection: by their series up to |x| = 1 (to x^11 and
 // x^12 in FP32: below 1e-9), where nearly all are
 __device__ __forceinline__ void m_sincos_small(float x, float *s, float *c) {
@@ -255,7 +359,29 @@ __device__ __forceinline__ void m_sincos_small(float x, float *s, float *c) {
     sincosf(x, s, c);
   }
 }
-__device__ __forceinline__ void m_sincos_small(double x, double *s, double *c) { sincos(x, s, c); }
+// (in FP64 up to 1/2, to x^15 and x^16: below 1e-18)
+__device__ __forceinline__ void m_sincos_small(double x, double *s, double *c) {
+  if ((__double2hiint(x) & 0x7fffffff) < 0x3fe00000) {
+    const double t = x * x;
+    double p = fma(t, -1.0 / 1307674368000.0, 1.0 / 6227020800.0);
+    p = fma(t, p, -1.0 / 39916800.0);
+    p = fma(t, p, 1.0 / 362880.0);
+    p = fma(t, p, -1.0 / 5040.0);
+    p = fma(t, p, 1.0 / 120.0);
+    p = fma(t, p, -1.0 / 6.0);
+    *s = fma(x * t, p, x);
+    double q = fma(t, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
+    q = fma(t, q, 1.0 / 479001600.0);
+    q = fma(t, q, -1.0 / 3628800.0);
+    q = fma(t, q, 1.0 / 40320.0);
+    q = fma(t, q, -1.0 / 720.0);
+    q = fma(t, q, 1.0 / 24.0);
+    q = fma(t, q, -0.5);
+    *c = fma(t, q, 1.0);
+  } else {
+    sincos(x, s, c);
+  }
+}
 
 // Sort key of cell (i, j, k): 4x4x4 tiles in x-fastest tile order, cells
 // x-fastest inside a tile, so consecutive electrons share a compact box.
@@ -310,6 +436,21 @@ __device__ __forceinline__ void rotate_near(R &dx, R &dy, R &dz, R ct, R st, R c
   dx = dx * k + qx;
   dy = dy * k + (up ? qy : -qy);
   dz = dz * ct - V;
+}
+
+// none of them infinite or NaN: zero times each is zero (in FP64 by the
+// exponents, off the FP64 unit)
+__device__ __forceinline__ bool all_finite(float a, float b, float c, float d, float e, float f,
+                                           float g) {
+  return 0.0f * a + 0.0f * b + 0.0f * c + 0.0f * d + 0.0f * e + 0.0f * f + 0.0f * g == 0.0f;
+}
+__device__ __forceinline__ bool all_finite(double a, double b, double c, double d, double e,
+                                           double f, double g) {
+  const int m = 0x7ff00000;
+  int x = max(__double2hiint(a) & m, __double2hiint(b) & m);
+  x = max(max(x, __double2hiint(c) & m), __double2hiint(d) & m);
+  x = max(max(x, __double2hiint(e) & m), max(__double2hiint(f) & m, __double2hiint(g) & m));
+  return x != m;
 }
 
 // ---------------------------------------------------------------- reductions

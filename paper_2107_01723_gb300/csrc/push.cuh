@@ -112,7 +112,7 @@ __device__ __forceinline__ R trilerp(const Grid<R> &g, int c, int b, R fx, R fy,
 // G(u0) = integral_{u0}^{1} s(u)/u du for s(u) = (4/3)(1-u) + u^2
 template <typename R>
 __device__ __forceinline__ R shape_G(R u0) {
-  return R(4.0 / 3.0) * (-m_flog(u0) - (R(1) - u0)) + R(0.5) * (R(1) - u0 * u0);
+  return R(4.0 / 3.0) * (-p_flog(u0) - (R(1) - u0)) + R(0.5) * (R(1) - u0 * u0);
 }
 
 // Photon energy from the inverse-CDF table (rows: ln eps, columns: the
@@ -388,7 +388,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
   } else if (K.physics & P_DRAG) {
     const R ig = m_rcp(gam);
     // ln(eps) + ln(gamma + 1)/2, and the bracket's terms in 1/gamma
-    const R br0 = R(0.5) * m_flog(eps * eps * (gam + R(1))) +
+    const R br0 = R(0.5) * p_flog(eps * eps * (gam + R(1))) +
                   ((R(0.909) * ig - R(0.818)) * ig - R(0.246));
     const R inv_beta = gam * inv;
     R de = R(0);
@@ -407,8 +407,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
       heat += w * de;
       eps = eps1;
       gam = R(1) + eps;
-      p = m_sqrt_near(eps * (gam + R(1)));
-      inv_p = m_rcp(p);
+      m_sqrt_both(eps * (gam + R(1)), p, inv_p);
     }
   }
 
@@ -419,16 +418,18 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
 #pragma unroll
     for (int s = 0; s < NS; ++s) {  // the elements' variances add
       if (NS > 1 && s >= h.n_solids) break;
-      R lg = m_flog(h.K_lg[s] * p);
+      R lg = p_flog(h.K_lg[s] * p);
       lg = lg < R(0) ? R(0) : lg;
       var += h.K_sc[s] * lg;
     }
     var *= gam * inv_p * (inv_p * inv_p);
     R s2, c2, st, ct;
     // Box-Muller normal deviate (its cosine changes only the deflection)
-    const R theta = m_sqrt(var * (R(-2) * m_log(unif<R>(r0.a)))) * m_fcos2pi(unif<R>(r0.b));
+    R normal;
+    p_cos_turn(r0.b, normal);
+    const R theta = m_sqrt(var * (R(-2) * p_log(unif<R>(r0.a)))) * normal;
     m_sincos_small(theta, &st, &ct);
-    m_sincos2pi(unif<R>(r0.c), &s2, &c2);
+    p_turn(r0.c, s2, c2);
     rotate_near(dx, dy, dz, ct, st, c2, s2);
   }
   if (K.physics & (P_DRAG | P_SCATTER)) {
@@ -813,8 +814,7 @@ __device__ __forceinline__ void push_warp(const Consts &K, const HotK<R> &h, con
   }
   if (in_range && id != kDead) {
     if (K.weighted) w = ld_stream(p.w + ip);  // uniform over the launch
-    // zero times each: NaN if any is infinite or NaN
-    if (R(0) * X + R(0) * Y + R(0) * Zc + R(0) * ux + R(0) * uy + R(0) * uz + R(0) * tau == R(0)) {
+    if (all_finite(X, Y, Zc, ux, uy, uz, tau)) {
       live = true;
     } else {
       if constexpr (SORT)
