@@ -1006,8 +1006,12 @@ int hpic_read_grid(hpic_ctx *ctx, int which, double *out) {
   const double *cells = cell_array(ctx, which);
   const void *src = cells;
   if (!cells || s != 1.0) {  // converted to double and scaled on the device
-    if (xfer_reserve(ctx, (size_t)L * sizeof(double)) != HPIC_OK) return read_grid_by_host(ctx, which, L, s, out);
-    double *d = static_cast<double *>(ctx->xfer);
+    // in the particle buffer that is not in use, if it is large enough
+    const size_t bytes = (size_t)L * sizeof(double);
+    const bool spare = bytes <= particle_bytes(ctx, ctx->stride);
+    if (!spare && xfer_reserve(ctx, bytes) != HPIC_OK)
+      return read_grid_by_host(ctx, which, L, s, out);
+    double *d = static_cast<double *>(spare ? ctx->pbuf[ctx->cur ^ 1] : ctx->xfer);
     const int grid = xfer_grid(ctx, L);
     if (cells)
       hpic::launch_scale_out<double>(cells, L, s, d, grid, ctx->stream);

@@ -14,12 +14,9 @@ struct Axis {
   R fN, fS;    // fractional offsets
 };
 
-// Linear weights along one axis; X in cells, in [0, n].  The half-staggered
-// lattice is held at its outermost value within half a cell of a wall.
-// The cell is read off the bits of X + 2^(p-1), p the significand's length,
-// added rounding down: no conversion instruction (a quarter-rate unit in FP32,
-// the FP64 unit in FP64), and the half-staggered offset is the other moved by
-// half a cell, exact in both (X >= 1 has no bits below half a cell's last).
+// The cell of X and the offset in it, by the bits of X + 2^(p-1), p the
+// significand's length, added rounding down: no conversion instruction (a
+// quarter-rate unit in FP32, the FP64 unit in FP64).
 __device__ __forceinline__ int cell_of(float X, float &f) {
   const float t = __fadd_rd(X, 8388608.0f);
   f = X - (t - 8388608.0f);
@@ -30,26 +27,44 @@ __device__ __forceinline__ int cell_of(double X, double &f) {
   f = X - (t - 4503599627370496.0);
   return __double2loint(t);
 }
-__device__ __forceinline__ bool upper_half(float f) { return f >= 0.5f; }
-__device__ __forceinline__ bool upper_half(double f) { return __double2hiint(f) >= 0x3fe00000; }
 
+// Linear weights along one axis; X in cells, in [0, n].  The half-staggered
+// lattice is held at its outermost value within half a cell of a wall.
+// FP64 reads the cell off the bits and moves its offset by half a cell for the
+// staggered one, exact as X >= 1 has no bits below half a cell's last: a third
+// of the FP64 operations.  FP32 converts: the selects cost more there (1e7
+// electrons 654 against 676 us, a batch of 8e6 713 against 732).
 template <typename R>
 __device__ __forceinline__ Axis<R> axis_weights(R X, int n) {
   Axis<R> a;
-  R f;
-  int i = cell_of(X, f);
-  if ((unsigned)i >= (unsigned)min(n, 1 << 22)) {  // the far wall itself, or a very long axis
-    i = min(max((int)m_floor(X), 0), n - 1);
-    f = X - R(i);
-  }
-  a.iN = i;
-  a.fN = f;
-  const bool up = upper_half(f);
-  a.iS = up ? i : i - 1;
-  a.fS = f + (up ? R(-0.5) : R(0.5));
-  if (a.iS < 0 || (up && i == n - 1)) {  // within half a cell of a wall
-    a.iS = i;
-    a.fS = R(0);
+  if constexpr (sizeof(R) == 8) {
+    R f;
+    int i = cell_of(X, f);
+    if ((unsigned)i >= (unsigned)n) {  // the far wall itself (or no position of the box)
+      i = min(max((int)m_floor(X), 0), n - 1);
+      f = X - R(i);
+    }
+    a.iN = i;
+    a.fN = f;
+    const bool up = __double2hiint(f) >= 0x3fe00000;  // f >= 1/2
+    a.iS = up ? i : i - 1;
+    a.fS = f + (up ? R(-0.5) : R(0.5));
+    if (a.iS < 0 || (up && i == n - 1)) {  // within half a cell of a wall
+      a.iS = i;
+      a.fS = R(0);
+    }
+  } else {
+    int i = (int)m_floor(X);
+    i = min(max(i, 0), n - 1);
+    a.iN = i;
+    a.fN = X - R(i);
+    R q = X - R(0.5);
+    q = q < R(0) ? R(0) : q;
+    q = q > R(n - 1) ? R(n - 1) : q;
+    int is = (int)m_floor(q);
+    is = min(max(is, 0), n - 1);
+    a.iS = is;
+    a.fS = q - R(is);
   }
   return a;
 }
@@ -353,93 +368,181 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
     Bz = trilerp(g, 5, g.node(ax.iS, ay.iS, az.iN), ax.fS, ay.fS, az.fN);
   }
 
-  // ---- Boris push: half kick, rotation, half kick
-  R gam;
-  const R eps0 = kinetic_near(ux * ux + uy * uy + uz * uz, gam);
-  {
-    const R mx = ux + R(0.5) * Ex, my = uy + R(0.5) * Ey, mz = uz + R(0.5) * Ez;
-    const R hh = R(0.5) * m_rsqrt(R(1) + mx * mx + my * my + mz * mz);
-    const R tx = Bx * hh, ty = By * hh, tz = Bz * hh;
-    const R s2 = R(2) * m_rcp(R(1) + tx * tx + ty * ty + tz * tz);
-    const R sx = tx * s2, sy_ = ty * s2, sz_ = tz * s2;
-    const R qx = mx + (my * tz - mz * ty), qy = my + (mz * tx - mx * tz), qz = mz + (mx * ty - my * tx);
-    ux = mx + (qy * sz_ - qz * sy_) + R(0.5) * Ex;
-    uy = my + (qz * sx - qx * sz_) + R(0.5) * Ey;
-    uz = mz + (qx * sy_ - qy * sx) + R(0.5) * Ez;
-  }
-  const R u2 = ux * ux + uy * uy + uz * uz;
-  R eps = kinetic_near(u2, gam);
-  acc.W += w * (eps0 - eps);
-  R heat = 0;
+  // Push, drag and scatter, in one of two forms.  FP64, and FP32 where there is
+  // no grid, hold the electron as direction and momentum, which saves roots,
+  // quotients and logarithms (FP64: 1e6 electrons 1670 -> 1290 us; FP32 in the
+  // unbounded medium 206 -> 195).  FP32 with the grid is held by the L1 data
+  // pipe and takes the same time either way (659 us at 1e7); it keeps the form
+  // whose every step is a rounded FP32 momentum, and with it the roundings of
+  // the runs already made.
+  constexpr bool kByDirection = sizeof(R) == 8 || FREE;
+  R eps, gam = R(0), p = R(0), heat = 0;
   bool alive = true;
-
-  // From here the electron is its direction d and its momentum p = |u|: the
-  // drag changes p alone and the scatter d alone, and the energy eps, gamma =
-  // 1 + eps and their reciprocals serve every term, so that no root or
-  // quotient is formed twice.  (u is rebuilt as p d after the collisions.)
-  const R inv = m_rsqrt_near(u2);
-  R p = u2 * inv, inv_p = inv;
-  R dx = ux * inv, dy = uy * inv, dz = uz * inv;
-
-  // ---- tracking cut and ionisation drag, Eq. (5)
-  if (eps < h.E_cut) {
-    heat += w * eps;
-    alive = false;
-  } else if (K.physics & P_DRAG) {
-    const R ig = m_rcp(gam);
-    // ln(eps) + ln(gamma + 1)/2, and the bracket's terms in 1/gamma
-    const R br0 = R(0.5) * p_flog(eps * eps * (gam + R(1))) +
-                  ((R(0.909) * ig - R(0.818)) * ig - R(0.246));
-    const R inv_beta = gam * inv;
-    R de = R(0);
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {  // the elements' stopping powers add
-      if (NS > 1 && s >= h.n_solids) break;  // constant indices: no local-memory copy
-      R br = br0 + h.L_I[s];
-      br = br < R(0) ? R(0) : br;
-      de += h.K_ion[s] * inv_beta * br;
+  if constexpr (kByDirection) {
+    // ---- Boris push: half kick, rotation, half kick
+    const R eps0 = kinetic_near(ux * ux + uy * uy + uz * uz, gam);
+    {
+      const R mx = ux + R(0.5) * Ex, my = uy + R(0.5) * Ey, mz = uz + R(0.5) * Ez;
+      const R hh = R(0.5) * m_rsqrt(R(1) + mx * mx + my * my + mz * mz);
+      const R tx = Bx * hh, ty = By * hh, tz = Bz * hh;
+      const R s2 = R(2) * m_rcp(R(1) + tx * tx + ty * ty + tz * tz);
+      const R sx = tx * s2, sy_ = ty * s2, sz_ = tz * s2;
+      const R qx = mx + (my * tz - mz * ty), qy = my + (mz * tx - mx * tz), qz = mz + (mx * ty - my * tx);
+      ux = mx + (qy * sz_ - qz * sy_) + R(0.5) * Ex;
+      uy = my + (qz * sx - qx * sz_) + R(0.5) * Ey;
+      uz = mz + (qx * sy_ - qy * sx) + R(0.5) * Ez;
     }
-    const R eps1 = eps - de;
-    if (eps1 < h.E_cut) {
+    const R u2 = ux * ux + uy * uy + uz * uz;
+    eps = kinetic_near(u2, gam);
+    acc.W += w * (eps0 - eps);
+
+    // From here the electron is its direction d and its momentum p = |u|: the
+    // drag changes p alone and the scatter d alone, and the energy eps, gamma =
+    // 1 + eps and their reciprocals serve every term, so that no root or
+    // quotient is formed twice.  (u is rebuilt as p d after the collisions.)
+    const R inv = m_rsqrt_near(u2);
+    R inv_p = inv;
+    p = u2 * inv;
+    R dx = ux * inv, dy = uy * inv, dz = uz * inv;
+
+    // ---- tracking cut and ionisation drag, Eq. (5)
+    if (eps < h.E_cut) {
       heat += w * eps;
       alive = false;
-    } else {
-      heat += w * de;
-      eps = eps1;
-      gam = R(1) + eps;
-      m_sqrt_both(eps * (gam + R(1)), p, inv_p);
-    }
-  }
-
-  // ---- Davies scatter, Eq. (B4): polar Gamma*sigma, azimuth uniform
-  if (alive && (K.physics & P_SCATTER)) {
-    const U4 r0 = philox10(sc.step, id, 0u, sc.target, sc.key0, sc.key1);
-    R var = R(0);
+    } else if (K.physics & P_DRAG) {
+      const R ig = m_rcp(gam);
+      // ln(eps) + ln(gamma + 1)/2, and the bracket's terms in 1/gamma
+      const R br0 = R(0.5) * p_flog(eps * eps * (gam + R(1))) +
+                    ((R(0.909) * ig - R(0.818)) * ig - R(0.246));
+      const R inv_beta = gam * inv;
+      R de = R(0);
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {  // the elements' variances add
-      if (NS > 1 && s >= h.n_solids) break;
-      R lg = p_flog(h.K_lg[s] * p);
-      lg = lg < R(0) ? R(0) : lg;
-      var += h.K_sc[s] * lg;
+      for (int s = 0; s < NS; ++s) {  // the elements' stopping powers add
+        if (NS > 1 && s >= h.n_solids) break;  // constant indices: no local-memory copy
+        R br = br0 + h.L_I[s];
+        br = br < R(0) ? R(0) : br;
+        de += h.K_ion[s] * inv_beta * br;
+      }
+      const R eps1 = eps - de;
+      if (eps1 < h.E_cut) {
+        heat += w * eps;
+        alive = false;
+      } else {
+        heat += w * de;
+        eps = eps1;
+        gam = R(1) + eps;
+        m_sqrt_both(eps * (gam + R(1)), p, inv_p);
+      }
     }
-    var *= gam * inv_p * (inv_p * inv_p);
-    R s2, c2, st, ct;
-    // Box-Muller normal deviate (its cosine changes only the deflection)
-    R normal;
-    p_cos_turn(r0.b, normal);
-    const R theta = m_sqrt(var * (R(-2) * p_log(unif<R>(r0.a)))) * normal;
-    m_sincos_small(theta, &st, &ct);
-    p_turn(r0.c, s2, c2);
-    rotate_near(dx, dy, dz, ct, st, c2, s2);
-  }
-  if (K.physics & (P_DRAG | P_SCATTER)) {
-    ux = p * dx; uy = p * dy; uz = p * dz;
+
+    // ---- Davies scatter, Eq. (B4): polar Gamma*sigma, azimuth uniform
+    if (alive && (K.physics & P_SCATTER)) {
+      const U4 r0 = philox10(sc.step, id, 0u, sc.target, sc.key0, sc.key1);
+      R var = R(0);
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {  // the elements' variances add
+        if (NS > 1 && s >= h.n_solids) break;
+        R lg = p_flog(h.K_lg[s] * p);
+        lg = lg < R(0) ? R(0) : lg;
+        var += h.K_sc[s] * lg;
+      }
+      var *= gam * inv_p * (inv_p * inv_p);
+      R s2, c2, st, ct;
+      // Box-Muller normal deviate (its cosine changes only the deflection)
+      R normal;
+      p_cos_turn(r0.b, normal);
+      const R theta = m_sqrt(var * (R(-2) * p_log(unif<R>(r0.a)))) * normal;
+      m_sincos_small(theta, &st, &ct);
+      p_turn(r0.c, s2, c2);
+      rotate_near(dx, dy, dz, ct, st, c2, s2);
+    }
+    if (K.physics & (P_DRAG | P_SCATTER)) {
+      ux = p * dx; uy = p * dy; uz = p * dz;
+    }
+  } else {
+    // ---- Boris push: half kick, rotation, half kick
+    const R eps0 = kinetic(ux, uy, uz);
+    {
+      const R mx = ux + R(0.5) * Ex, my = uy + R(0.5) * Ey, mz = uz + R(0.5) * Ez;
+      const R gm = m_sqrt(R(1) + mx * mx + my * my + mz * mz);
+      const R hh = R(0.5) / gm;
+      const R tx = Bx * hh, ty = By * hh, tz = Bz * hh;
+      const R s2 = R(2) / (R(1) + tx * tx + ty * ty + tz * tz);
+      const R sx = tx * s2, sy_ = ty * s2, sz_ = tz * s2;
+      const R qx = mx + (my * tz - mz * ty), qy = my + (mz * tx - mx * tz), qz = mz + (mx * ty - my * tx);
+      ux = mx + (qy * sz_ - qz * sy_) + R(0.5) * Ex;
+      uy = my + (qz * sx - qx * sz_) + R(0.5) * Ey;
+      uz = mz + (qx * sy_ - qy * sx) + R(0.5) * Ez;
+    }
+    eps = kinetic(ux, uy, uz);
+    acc.W += w * (eps0 - eps);
+
+    // ---- tracking cut and ionisation drag, Eq. (5)
+    if (eps < h.E_cut) {
+      heat += w * eps;
+      alive = false;
+    } else if (K.physics & P_DRAG) {
+      const R gam = R(1) + eps;
+      const R beta = u_of_eps(eps) / gam;
+      const R ig = R(1) / gam;
+      const R le = m_flog(eps), lh = R(0.5) * m_flog(gam + R(1));
+      const R a2 = R(0.909) * ig * ig, a1 = R(0.818) * ig;
+      R de = R(0);
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {  // the elements' stopping powers add
+        if (NS > 1 && s >= h.n_solids) break;  // constant indices: no local-memory copy
+        R br = le + h.L_I[s] + lh + a2 - a1 - R(0.246);
+        br = br < R(0) ? R(0) : br;
+        de += h.K_ion[s] / beta * br;
+      }
+      const R eps1 = eps - de;
+      if (eps1 < h.E_cut) {
+        heat += w * eps;
+        alive = false;
+      } else {
+        const R s = m_div_rn(u_of_eps(eps1), m_sqrt_rn(ux * ux + uy * uy + uz * uz));
+        ux *= s; uy *= s; uz *= s;
+        heat += w * de;
+        eps = eps1;
+      }
+    }
+
+    // ---- Davies scatter, Eq. (B4): polar Gamma*sigma, azimuth uniform
+    if (alive && (K.physics & P_SCATTER)) {
+      const U4 r0 = philox10(sc.step, id, 0u, sc.target, sc.key0, sc.key1);
+      const R u2 = ux * ux + uy * uy + uz * uz;
+      const R inv = m_rsqrt_rn(u2);
+      const R un = u2 * inv;
+      const R gam = m_sqrt(R(1) + u2);
+      R var = R(0);
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {  // the elements' variances add
+        if (NS > 1 && s >= h.n_solids) break;
+        R lg = m_flog(h.K_lg[s] * un);
+        lg = lg < R(0) ? R(0) : lg;
+        var += h.K_sc[s] * gam / (un * un * un) * lg;
+      }
+      const R sig = m_sqrt(var);
+      R s2, c2, st, ct;
+      // Box-Muller normal deviate (its cosine changes only the deflection)
+      const R gauss = m_sqrt(R(-2) * m_log(unif<R>(r0.a))) * m_fcos2pi(unif<R>(r0.b));
+      m_sincos(gauss * sig, &st, &ct);
+      m_sincos2pi(unif<R>(r0.c), &s2, &c2);
+      R dx = ux * inv, dy = uy * inv, dz = uz * inv;
+      rotate(dx, dy, dz, ct, st, c2, s2);
+      ux = un * dx; uy = un * dy; uz = un * dz;
+    }
   }
 
   // ---- bremsstrahlung by optical depth (App. B)
   if (alive && (K.physics & P_BREM) && eps > h.k_min) {
-    const R inv_eps = m_rcp(eps);
-    R dtau = h.K_tau * (p * inv_eps) * shape_G(h.k_min * inv_eps);
+    R dtau;
+    if constexpr (kByDirection) {
+      const R inv_eps = m_rcp(eps);
+      dtau = h.K_tau * (p * inv_eps) * shape_G(h.k_min * inv_eps);
+    } else {
+      dtau = h.K_tau * u_of_eps(eps) / eps * shape_G(h.k_min / eps);
+    }
     if (K.physics & P_FSIGMA) dtau *= __ldg(g.Fsig + ax.iN + nx * (ay.iN + ny * az.iN));
     tau -= dtau;
     if (tau <= R(0)) {
@@ -473,9 +576,9 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
   }
 
   // ---- move, then escape or reflux at each face crossed (out of line: rare)
-  ig = m_rcp(gam);
-  const R cdt = ig * h.cdt;
-  R pos[3] = {X + ux * cdt, Y + uy * cdt, Zc + uz * cdt};
+  if constexpr (kByDirection) ig = m_rcp(gam);
+  else ig = R(1) / m_sqrt(R(1) + ux * ux + uy * uy + uz * uz);
+  R pos[3] = {X + ux * ig * h.cdt, Y + uy * ig * h.cdt, Zc + uz * ig * h.cdt};
   if (!unbounded && !(pos[0] >= R(0) && pos[0] <= R(nx) && pos[1] >= R(0) && pos[1] <= R(ny) &&
                       pos[2] >= R(0) && pos[2] <= R(nz))) {
     const Crossing<R> c = cross_faces<R>(h.eps_esc, h.du_reflux, h.sigma_dtheta, sc.step,
@@ -489,7 +592,8 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
     if (!c.alive) return false;
     pos[0] = c.pos[0]; pos[1] = c.pos[1]; pos[2] = c.pos[2];
     ux = c.u[0]; uy = c.u[1]; uz = c.u[2];
-    ig = m_rsqrt(R(1) + ux * ux + uy * uy + uz * uz);
+    if constexpr (kByDirection) ig = m_rsqrt(R(1) + ux * ux + uy * uy + uz * uz);
+    else ig = R(1) / m_sqrt(R(1) + ux * ux + uy * uy + uz * uz);
   }
   X = pos[0]; Y = pos[1]; Zc = pos[2];
 
