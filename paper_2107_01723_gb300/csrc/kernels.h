@@ -220,6 +220,16 @@ template <typename R>
 constexpr int push_threads(int mode) {
   return sizeof(R) == 4 ? (mode == kPushFree ? 512 : 384) : 256;
 }
+// Slots that fill less than kPushFewWaves such waves are pushed by as many
+// warps in blocks of kPushFewThreads instead: the scheduler deals them out over
+// all SMs, where the large blocks of a partial wave fill some SMs and leave the
+// others idle.  k_push in us, large blocks -> 64 threads (32), gold 64^3, FP32:
+// 1e5 electrons 24.1 -> 19.0 (19.4), 3e5 38.8 -> 33.9 (35.9), 8e5 68.5 -> 62.0
+// (74.6), 1.5e6 107.7 -> 105.9; FP64: 2e4 66.7 -> 52.8 (49.8), 1e5 157 -> 147
+// (145), 2e5 278 -> 252, 5e5 592 -> 562.  Beyond about eight waves the twelve
+// warps of a large block gain more from the L1 lines that they share: 1e7 655
+// (64 threads: 661), an unbounded 8e6 144 (150), FP64 1e6 level.
+constexpr int kPushFewThreads = 64, kPushFewWaves = 8;
 // resident 256-thread blocks per SM of the field and heating kernels (their
 // launch bounds); they are launched as one wave of sm_count times this many
 // blocks (grid-stride over the nodes), so no partial second wave trails.  Four

@@ -31,8 +31,8 @@ namespace hpic {
 // medium; the other modes' code is compiled out.
 template <typename R, int NS, int MODE>
 // Launched as one persistent wave in the shape push_threads/push_blocks_per_sm
-// give: the kernel is issue- and latency-bound and gains from the warps, up
-// to the register count at which spills begin.
+// give, or with as many warps in smaller blocks (kPushFewThreads); FP32 gains
+// from the warps up to the register count at which spills begin.
 __global__ void __launch_bounds__(push_threads<R>(MODE), push_blocks_per_sm<R>(MODE))
 k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__restrict__ tab,
        Counters *cnt, TallyView tv, const SortOut<R> so, const KeyOut<R> ko) {
@@ -223,8 +223,8 @@ __global__ void k_advance(const StepEnd end) {
 // ---------------------------------------------------------------- launchers
 
 template <typename R, int MODE>
-constexpr size_t push_stage_bytes() {
-  return (push_threads<R>(MODE) / 32) * push_warp_words<R, MODE>() * sizeof(R);
+constexpr size_t push_stage_bytes(int threads = push_threads<R>(MODE)) {
+  return (threads / 32) * push_warp_words<R, MODE>() * sizeof(R);
 }
 
 cudaError_t prepare_push() {
@@ -252,12 +252,14 @@ template <typename R, int NS, int MODE>
 void launch_push_mode(const Consts &K, const HotK<R> &h, PView<R> p, GView<R> g, const R *table,
                       Counters *cnt, TallyView tv, long long cap, int sm_count, cudaStream_t st,
                       const SortOut<R> &so, const KeyOut<R> &ko) {
-  // one resident wave, or the blocks the slots fill
-  constexpr int threads = push_threads<R>(MODE);
-  const long long want = (cap + threads - 1) / threads;
-  const long long wave = (long long)sm_count * push_blocks_per_sm<R>(MODE);
+  // one resident wave, or the blocks the slots fill (small ones where these are
+  // few: kernels.h)
+  constexpr int full = push_threads<R>(MODE);
+  const long long warps = (long long)sm_count * push_blocks_per_sm<R>(MODE) * (full / 32);
+  const int threads = (cap + 31) / 32 < kPushFewWaves * warps ? kPushFewThreads : full;
+  const long long want = (cap + threads - 1) / threads, wave = warps / (threads / 32);
   const int grid = (int)(want < wave ? want : wave);
-  constexpr size_t smem = push_stage_bytes<R, MODE>();
+  const size_t smem = push_stage_bytes<R, MODE>(threads);
   if (MODE == kPushSort)  // it follows the sort's scan
     launch_chained(k_push<R, NS, MODE>, grid, threads, smem, st, K, h, p, g, table, cnt, tv, so, ko);
   else
