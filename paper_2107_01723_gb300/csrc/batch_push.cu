@@ -4,8 +4,8 @@
 // Every target owns a fixed range of slots in one shared structure of
 // arrays.  Per step a one-block plan turns the targets' live counts into a
 // prefix of warp-sized tasks (32 consecutive slots of one target); the
-// persistent push kernel's warps take tasks in a global sweep (task w,
-// w + all warps, ...), so at any moment the whole GPU works on a narrow
+// persistent push kernel's warps take tasks in a global sweep (each its first
+// task, then that many warps on, ...), so at any moment the whole GPU works on a narrow
 // window of slots and each target's grid stays hot in L2 while it is swept.
 // A warp meets each target once per sweep: it then copies the target's
 // constants into shared memory and, when it moves on, adds its tally sums to
@@ -18,8 +18,8 @@ namespace hpic {
 
 // Threads per block of the persistent push, by precision and blocks per SM
 // (MINB): FP32 runs 512 at two blocks per SM (64 registers) and 384 at three
-// (56 registers), 256 otherwise; FP64 runs 256.  A block's warps take
-// consecutive tasks, so larger blocks share more of their gathers' L1 lines
+// (56 registers), 256 otherwise; FP64 runs 256.  Where a block's
+// warps take consecutive tasks, larger blocks share more of their gathers' L1 lines
 // (the single-target kernel measured three blocks of 384 3.4 % faster than
 // five of 256 at 48 registers).
 // One definition serves the kernels' launch bounds, the launches and the
@@ -31,10 +31,25 @@ __host__ __device__ constexpr int batch_threads_for(bool fp32, int blocks_per_sm
 template <typename R, int MINB>
 __host__ __device__ constexpr int batch_threads() { return batch_threads_for(sizeof(R) == 4, MINB); }
 constexpr int kBatchMaxWarps = 16;
+// Tasks are dealt to the blocks in pairs (two neighbouring tasks to a block,
+// the next two to the next block), so a partial sweep, or a whole step of few
+// electrons, occupies all SMs: with a block's warps on consecutive tasks, the
+// tasks of 3e4 electrons sat on 59 of the 152 SMs.  k_batch_push in us,
+// consecutive -> pairs (single tasks; fours), 8 targets, FP32 at two blocks per
+// SM: 1.5e5 electrons 43.4 -> 31.9 (32.9; 34.1), 6e5 84.7 -> 76.2, 2e6 193 -> 186,
+// 8e6 625 -> 621; 16 targets of 8e6 in all 715 -> 702; FP64: 3e4 103 -> 59 (57;
+// 64), 5e5 588 -> 562.  Blocks of 12 warps and fewer gain up to about eight
+// sweeps (1.5e5 45.1 -> 34.4, 1.2e6 136 -> 133) and are mixed beyond (2e6 194 ->
+// 199, 3e6 in 16 targets 343 -> 334, 8e6 651 -> 653): there they take
+// consecutive tasks.
+constexpr int kBatchDeal = 2, kBatchFewSweeps = 8;
 static_assert(batch_threads_for(true, 2) / 32 <= kBatchMaxWarps &&
                   batch_threads_for(true, 3) / 32 <= kBatchMaxWarps &&
                   batch_threads_for(false, 2) / 32 <= kBatchMaxWarps,
               "the largest block's stages are what the shared-memory limit is set for");
+static_assert(batch_threads_for(true, 5) % (32 * kBatchDeal) == 0 &&
+                  batch_threads_for(true, 3) % (32 * kBatchDeal) == 0,
+              "a block's warps are whole pairs");
 static_assert(batch_threads_for(true, 1) == batch_threads_for(true, 2),
               "one block per SM in FP32 runs the two-block kernel");
 
@@ -109,7 +124,12 @@ k_batch_push(const Consts Krun, const BatchItem<R> *__restrict__ items, BatchDev
   TargetHot<R> &it = wc[warp];
   int t = -1;
   Acc<R> acc;
-  for (long long w = blockIdx.x * (long long)kBatchWarps + warp; w < ntask; w += nwarps) {
+  // the task order: see kBatchDeal
+  const bool deal = kBatchWarps >= 16 || ntask < kBatchFewSweeps * nwarps;
+  const long long first =
+      deal ? (warp / kBatchDeal * (long long)gridDim.x + blockIdx.x) * kBatchDeal + warp % kBatchDeal
+           : blockIdx.x * (long long)kBatchWarps + warp;
+  for (long long w = first; w < ntask; w += nwarps) {
     int tn = t < 0 ? 0 : t;
     while (wpref_s[tn + 1] <= w) ++tn;
     if (tn != t) {  // warp-uniform: a new target
