@@ -70,7 +70,7 @@ k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__rest
 
   // Each warp's four sums, one shared add each.  (A block-wide FP64 tree over
   // all thirteen slots, in every block of the wave, cost 65 FP64 adds per warp:
-  // a launch over 1e5 electrons took 24.5 us, now 20.8 us.)
+  // a launch over 1e5 electrons took 24.5 us, without it 20.8 us.)
   acc.flush_warp(sums);
   __syncthreads();
   if (threadIdx.x < kAccN && sums[threadIdx.x] != 0.0)
