@@ -571,8 +571,8 @@ void *device_address(const void *p, size_t bytes) {
 // Gives every page of a pageable host array its memory before the device's copy
 // arrives there (the contents stay).  A copy into pages that have none yet faults
 // them in from the device's side, which in three processes of five took 14 to 28
-// ms for a grid of 33 MB (with the touch, 0.2 in five of five; pages that are
-// present cost 0.01 ms).
+// ms for a grid of 33 MB (with the touch, 0.2 in five of five, 10 in one other;
+// pages that are present cost 0.01 ms).
 void touch_pages(void *p, size_t bytes) {
   static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
   volatile char *c = static_cast<volatile char *>(p);

@@ -838,8 +838,8 @@ __device__ __forceinline__ void st_stream(R *p, R v) { __stcs(p, v); }
 // lane) while the warp works on the present ones.  Used in the unbounded
 // medium in FP32 (kPushFree), where DRAM latency took a third of the warps'
 // time and there is no deposit stage: 2^23 electrons 195 -> 154 us (2.6 ->
-// 3.3 TB/s), of which the copies 10 us and the rest 48 warps per SM at 40
-// registers, for 36 at 56.
+// 3.3 TB/s; since the deviates' own work shrank 144 us, 3.5 TB/s), of which the
+// copies 10 us and the rest 48 warps per SM at 40 registers, for 36 at 56.
 // (With the grid on, it costs: the kernel is then held by the L1 data pipe,
 // 75 % busy, and the copies pass through it twice: 659 -> 690 us at 1e7.)
 template <typename R, int MODE>
