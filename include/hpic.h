@@ -272,8 +272,8 @@ int hpic_count_particles(hpic_ctx *ctx, int64_t *n);
  * may be NULL (that array is skipped).  The compaction and the conversion
  * to double run on the device, through a scratch buffer the context owns
  * (grown to 8 bytes per electron slot, and by hpic_read_grid to 8 bytes per
- * node of a grid larger than the particle storage, where it can be had; freed
- * by hpic_destroy or hpic_batch_destroy);
+ * node of a batch target's grid or of one larger than the particle storage,
+ * where it can be had; freed by hpic_destroy or hpic_batch_destroy);
  * HPIC_ENOMEM if it cannot be allocated.  This call and hpic_load_particles /
  * hpic_count_particles synchronise the stream.  The host arrays here and in
  * hpic_load_particles may be page-locked (cudaHostAlloc) or pageable, each for

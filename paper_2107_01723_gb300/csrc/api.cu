@@ -1021,9 +1021,11 @@ int hpic_read_grid(hpic_ctx *ctx, int which, double *out) {
   const double *cells = cell_array(ctx, which);
   const void *src = cells;
   if (!cells || s != 1.0) {  // converted to double and scaled on the device
-    // in the particle buffer that is not in use, if it is large enough
+    // in the particle buffer that is not in use, if it is this context's alone
+    // (a batch's targets share one, and each may be read by its own thread) and
+    // large enough
     const size_t bytes = (size_t)L * sizeof(double);
-    const bool spare = bytes <= particle_bytes(ctx, ctx->stride);
+    const bool spare = !ctx->owner && bytes <= particle_bytes(ctx, ctx->stride);
     if (!spare && xfer_reserve(ctx, bytes) != HPIC_OK)
       return read_grid_by_host(ctx, which, L, s, out);
     double *d = static_cast<double *>(spare ? ctx->pbuf[ctx->cur ^ 1] : ctx->xfer);
