@@ -279,7 +279,9 @@ int hpic_count_particles(hpic_ctx *ctx, int64_t *n);
  * hpic_load_particles may be page-locked (cudaHostAlloc) or pageable, each for
  * itself; page-locked ones, allocated once and reused, are written and read
  * by the device across the link, all arrays in one kernel, without the
- * driver's staging copies and the page faults of fresh memory. */
+ * driver's staging copies and the page faults of fresh memory.  (A page-locked
+ * array that does not start at a multiple of its element's size is copied like
+ * a pageable one.) */
 int hpic_read_particles(hpic_ctx *ctx, double *x, double *y, double *z,
                         double *ux, double *uy, double *uz, double *tau,
                         uint32_t *id, int64_t cap, int64_t *n);

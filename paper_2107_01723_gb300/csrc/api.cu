@@ -551,9 +551,12 @@ int xfer_grid(const hpic_ctx *ctx, long long n) {
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
-// The device's address of `bytes` of page-locked host memory at p, or NULL
-// where it is not (pageable memory is copied through the driver).
-void *device_address(const void *p, size_t bytes) {
+// The device's address of `bytes` of page-locked host memory at p, of elements of
+// `size` bytes, or NULL where kernels cannot use it: pageable memory, and arrays
+// that do not start at a multiple of their element (a block that holds arrays of
+// several types, one behind the other).  Those are copied through the driver.
+void *device_address(const void *p, size_t bytes, size_t size) {
+  if (reinterpret_cast<uintptr_t>(p) % size) return nullptr;
   cudaPointerAttributes a{}, z{};
   const char *end = static_cast<const char *>(p) + (bytes ? bytes - 1 : 0);
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
@@ -562,10 +565,16 @@ void *device_address(const void *p, size_t bytes) {
     return nullptr;
   }
   if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer ||
+      reinterpret_cast<uintptr_t>(a.devicePointer) % size ||
       static_cast<char *>(z.devicePointer) - static_cast<char *>(a.devicePointer) !=
           end - static_cast<const char *>(p))
     return nullptr;
   return a.devicePointer;
+}
+// of n elements of T
+template <typename T>
+T *device_array(T *p, long long n) {
+  return static_cast<T *>(device_address(p, (size_t)n * sizeof(T), sizeof(T)));
 }
 
 // Gives every page of a pageable host array its memory before the device's copy
@@ -612,10 +621,10 @@ int read_particles_impl(hpic_ctx *ctx, double *x, double *y, double *z, double *
   hpic::ParticleOut direct{};
   bool any = false;
   for (int q = 0; q < 7; ++q) {
-    if (dst[q]) direct.a[q] = static_cast<double *>(device_address(dst[q], live * sizeof(double)));
+    if (dst[q]) direct.a[q] = device_array(dst[q], live);
     any |= direct.a[q] != nullptr;
   }
-  if (id) direct.id = static_cast<uint32_t *>(device_address(id, live * sizeof(uint32_t)));
+  if (id) direct.id = device_array(id, live);
   if (any || direct.id) hpic::launch_read_out<R>(P, n, cc, dx, direct, ctx->stream);
   for (int q = 0; q < 8; ++q) {
     void *to = q < 7 ? static_cast<void *>(dst[q]) : id;
@@ -652,11 +661,11 @@ int load_particles_impl(hpic_ctx *ctx, int64_t n, const double *x, const double 
   bool staged = false, any = false;
   if (n > 0) {
     for (int q = 0; q < 7; ++q) {
-      direct.a[q] = static_cast<const double *>(device_address(src[q], n * sizeof(double)));
+      direct.a[q] = device_array(src[q], n);
       staged |= !direct.a[q];
       any |= direct.a[q] != nullptr;
     }
-    direct.id = static_cast<const uint32_t *>(device_address(id, n * sizeof(uint32_t)));
+    direct.id = device_array(id, n);
     staged |= !direct.id;
   }
   const size_t data_off = 256;  // the error count first
