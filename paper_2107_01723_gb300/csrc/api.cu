@@ -1,6 +1,7 @@
 // Host side of the C-ABI in include/hpic.h: context, device buffers, the
 // folding of the paper's SI coefficients into normalised kernel constants,
 // and the per-step launch sequence.
+#include <cuda.h>
 #include <unistd.h>
 
 #include <cmath>
@@ -42,6 +43,7 @@ int fail(hpic_ctx *c, int code, const std::string &msg) {
 }
 
 int cuda_fail(hpic_ctx *c, cudaError_t e, const char *where) {
+  cudaGetLastError();  // reported here, not by the next call as well
   return fail(c, HPIC_ECUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
@@ -551,23 +553,44 @@ int xfer_grid(const hpic_ctx *ctx, long long n) {
   return (int)(want < 1 ? 1 : (want < cap ? want : cap));
 }
 
+// The driver's cuPointerGetAttribute (this library links the runtime alone), or
+// NULL where it cannot be had.
+using PointerAttribute = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
+PointerAttribute pointer_attribute() {
+  static const PointerAttribute get = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000,
+                                                           cudaEnableDefault, &found);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && found == cudaDriverEntryPointSuccess
+               ? reinterpret_cast<PointerAttribute>(f) : nullptr;
+  }();
+  return get;
+}
+
 // The device's address of `bytes` of page-locked host memory at p, of elements of
-// `size` bytes, or NULL where kernels cannot use it: pageable memory, and arrays
-// that do not start at a multiple of their element (a block that holds arrays of
-// several types, one behind the other).  Those are copied through the driver.
+// `size` bytes, or NULL where kernels cannot use it: pageable memory, an array that
+// reaches beyond one allocation or registration (what lies between two of them may
+// be pageable), and arrays that do not start at a multiple of their element (a block
+// that holds arrays of several types, one behind the other).  Those are copied
+// through the driver.
 void *device_address(const void *p, size_t bytes, size_t size) {
-  if (reinterpret_cast<uintptr_t>(p) % size) return nullptr;
-  cudaPointerAttributes a{}, z{};
-  const char *end = static_cast<const char *>(p) + (bytes ? bytes - 1 : 0);
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-      cudaPointerGetAttributes(&z, end) != cudaSuccess) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+  cudaPointerAttributes a{};
+  if (at % size || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer ||
-      reinterpret_cast<uintptr_t>(a.devicePointer) % size ||
-      static_cast<char *>(z.devicePointer) - static_cast<char *>(a.devicePointer) !=
-          end - static_cast<const char *>(p))
+  if (a.type != cudaMemoryTypeHost || !a.devicePointer ||
+      reinterpret_cast<uintptr_t>(a.devicePointer) % size)
+    return nullptr;
+  const PointerAttribute get = pointer_attribute();
+  CUdeviceptr start = 0;
+  size_t length = 0;
+  if (!get || get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+      get(&length, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS || at < start ||
+      at - start > length || bytes > length - (at - start))
     return nullptr;
   return a.devicePointer;
 }

@@ -47,3 +47,40 @@ def test_arrays_at_any_byte(precision, offset):
         for k in KEYS:  # cells and back: two roundings in double of an FP32 value
             assert np.max(np.abs(got[k] - p[k])) <= 4e-16 * np.max(np.abs(p[k])), k
     s.close()
+
+
+def test_array_across_two_registrations():
+    """Arrays whose two ends are page-locked and whose middle is not: the ends alone do
+    not make them page-locked.  They are copied, or the copy is refused with a status."""
+    import torch
+    rt = torch.cuda.cudart()
+    torch.cuda.init()
+    page = 1 << 16
+    n = 3 * page // 8
+    t = W.target(n=(9, 12, 10))
+    raw = np.empty(8 * 4 * page, np.uint8)
+    base = -raw.ctypes.data % page
+    rng = np.random.default_rng(2)
+    p = {k: rng.uniform(0.1, 0.9, n) * t[m] * t["dx"] for k, m in zip("xyz", ("nx", "ny", "nz"))}
+    p.update({k: rng.normal(size=n) for k in ("ux", "uy", "uz")})
+    p["tau"] = rng.exponential(1.0, n)
+    p["id"] = np.arange(n, dtype=np.uint32)
+    given = dict(p, x=np.frombuffer(raw.data, np.float64, n, base))
+    given["x"][:] = p["x"]
+    first = raw.ctypes.data + base
+    for at in (first, first + 2 * page):
+        assert int(rt.cudaHostRegister(at, page, 0)) == 0
+    try:
+        s = hpic.Sim(t, None, W.run(), precision=hpic.HPIC_FP64)
+        s.set_particles(p)
+        want = s.particles()
+        try:
+            s.set_particles(given)
+        except hpic.HpicError as e:
+            assert e.code == hpic.HPIC_ECUDA
+        got = s.particles()
+        assert all(np.array_equal(got[k], want[k]) for k in KEYS + ("id",))
+        s.close()
+    finally:
+        for at in (first, first + 2 * page):
+            rt.cudaHostUnregister(at)
