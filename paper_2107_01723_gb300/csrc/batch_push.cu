@@ -166,7 +166,7 @@ k_batch_push(const Consts Krun, const BatchItem<R> *__restrict__ items, BatchDev
     const long long local = (w - wpref_s[t]) * 32 + lane;
     push_warp<R, NS, SORT ? kPushSort : kPushPlain>(
         Krun, it.h, it.grid, tab, it.tv, sc, p, it.off + local, local < it.n, acc,
-        tal_s + t * kAccN, stage, -1, SORT ? &so : nullptr, SORT ? &it.sshift : nullptr, nullptr);
+        tal_s + t * kAccN, stage, SORT ? &so : nullptr, SORT ? &it.sshift : nullptr, nullptr);
   }
   if (t >= 0) acc.flush_warp(tal_s + t * kAccN);
   __syncthreads();

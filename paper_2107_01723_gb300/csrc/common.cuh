@@ -201,54 +201,30 @@ __device__ __forceinline__ double min_positive(double a, double b) {
   return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
 }
 
-// Reciprocals and roots for the per-electron arithmetic, of normal numbers
-// well inside FP32's range (others take the plain expressions in FP64; in
-// FP32 callers keep to x > 0).
-// FP32: the hardware estimate (m_rcp, m_rsqrt: 1-2 ulp), or one Newton step on
-// its residual formed with a fused multiply-add (m_*_near: the rounded result
-// but for rare last bits, without the range tests of the rounded functions),
-// where no rounding bias may enter an energy that no tally records.
-// FP64: from the FP32 estimate by one step of the series in the residual e
-// (about 1e-7), to e^2: three operations for 1/x, five for x^(-1/2), of a unit
-// that completes two per clock and SM.
+// FP64 reciprocals and roots for the per-electron arithmetic, of positive normal
+// numbers well inside FP32's range (others take the plain expressions): from the
+// FP32 estimate by one step of the series in the residual e (about 1e-7), to e^2:
+// three operations for 1/x, five for x^(-1/2), of a unit that completes two per
+// clock and SM.
 __device__ __forceinline__ bool fp32_range(double x) {  // [2^-100, 2^100)
   return (unsigned)(__double2hiint(x) - 0x39b00000) < 0x0c800000u;
 }
-__device__ __forceinline__ float m_rcp(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double m_rcp(double x) {
   if (!fp32_range(x)) return 1.0 / x;
   const double y = widen(__fdividef(1.0f, narrow(x)));
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ float m_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double m_rsqrt(double x) {
   if (!fp32_range(x)) return rsqrt(x);
   const double y = widen(rsqrtf(narrow(x)));
   const double e = fma(-x * y, y, 1.0);
   return fma(y, e * fma(0.375, e, 0.5), y);
 }
-__device__ __forceinline__ float m_rsqrt_near(float x) {
-  const float r = rsqrtf(x);
-  return fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
-}
 __device__ __forceinline__ double m_rsqrt_near(double x) { return m_rsqrt(x); }
-__device__ __forceinline__ float m_sqrt_near(float x) {
-  const float r = rsqrtf(x), s = x * r;
-  return fmaf(fmaf(-s, s, x), 0.5f * r, s);
-}
 __device__ __forceinline__ double m_sqrt_near(double x) { return x * m_rsqrt(x); }
-__device__ __forceinline__ float m_div_near(float n, float d) {
-  const float y = __fdividef(1.0f, d), q = n * y;
-  return fmaf(fmaf(-q, d, n), y, q);
-}
 __device__ __forceinline__ double m_div_near(double n, double d) { return n * m_rcp(d); }
-// p = sqrt(x) near-rounded, and 1/p
-__device__ __forceinline__ void m_sqrt_both(float x, float &p, float &inv) {
-  inv = rsqrtf(x);
-  const float s = x * inv;
-  p = fmaf(fmaf(-s, s, x), 0.5f * inv, s);
-}
+// p = sqrt(x) and 1/p
 __device__ __forceinline__ void m_sqrt_both(double x, double &p, double &inv) {
   inv = m_rsqrt(x);
   p = x * inv;
@@ -325,41 +301,18 @@ __device__ __forceinline__ void table_turn(uint32_t x, double &s, double &c) {
 }
 
 // the push's logarithms: of a deviate, and the quick one
-__device__ __forceinline__ float p_log(float x) { return logf(x); }
 __device__ __forceinline__ double p_log(double x) { return table_log(x); }
-__device__ __forceinline__ float p_flog(float x) { return __logf(x); }
+__device__ __forceinline__ float p_flog(float x) { return m_flog(x); }
 __device__ __forceinline__ double p_flog(double x) { return table_log(x); }
 // sine and cosine of the deviate x of the circle; its cosine for a normal deviate
-__device__ __forceinline__ void p_turn(uint32_t x, float &s, float &c) {
-  m_sincos2pi(unif<float>(x), &s, &c);
-}
 __device__ __forceinline__ void p_turn(uint32_t x, double &s, double &c) { table_turn(x, s, c); }
-__device__ __forceinline__ void p_cos_turn(uint32_t x, float &c) { c = m_fcos2pi(unif<float>(x)); }
 __device__ __forceinline__ void p_cos_turn(uint32_t x, double &c) {
   double s;
   table_turn(x, s, c);
 }
 
-// sine and cosine of a deflection: by their series up to |x| = 1 (to x^11 and
-// x^12 in FP32: below 1e-9), where nearly all are
-__device__ __forceinline__ void m_sincos_small(float x, float *s, float *c) {
-  if (fabsf(x) <= 1.0f) {
-    const float t = x * x;
-    float p = fmaf(t, -1.0f / 39916800.0f, 1.0f / 362880.0f);
-    p = fmaf(t, p, -1.0f / 5040.0f);
-    p = fmaf(t, p, 1.0f / 120.0f);
-    p = fmaf(t, p, -1.0f / 6.0f);
-    *s = fmaf(x * t, p, x);
-    float q = fmaf(t, -1.0f / 3628800.0f, 1.0f / 40320.0f);
-    q = fmaf(t, q, -1.0f / 720.0f);
-    q = fmaf(t, q, 1.0f / 24.0f);
-    q = fmaf(t, q, -0.5f);
-    *c = fmaf(t, q, 1.0f);
-  } else {
-    sincosf(x, s, c);
-  }
-}
-// (in FP64 up to 1/2, to x^15 and x^16: below 1e-18)
+// sine and cosine of a deflection: by their series up to |x| = 1/2 (to x^15 and
+// x^16: below 1e-18), where nearly all are
 __device__ __forceinline__ void m_sincos_small(double x, double *s, double *c) {
   if ((__double2hiint(x) & 0x7fffffff) < 0x3fe00000) {
     const double t = x * x;

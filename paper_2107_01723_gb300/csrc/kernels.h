@@ -207,19 +207,16 @@ std::vector<InjCell> injection_cells(const hpic_target_desc &t, const hpic_laser
 // warps take consecutive slots, so their gathers share L1 lines.  (Against
 // it: five blocks of 256 at 48 registers, 84 B of spills, 3.5 % slower; six
 // of 192 at 56 registers 3.2 %; four of 288 1.2 %; two of 576 level.)  FP64:
-// two blocks of 256.  In the unbounded medium FP32 runs three blocks of 512.
+// two blocks of 256.
 enum PushMode {
   kPushPlain = 0,  // a plain step
   kPushKeys = 1,   // one that also computes the next sort's keys (KeyOut)
-  kPushSort = 2,   // one that also sorts (SortOut)
-  kPushFree = 3    // a plain step in an unbounded medium: no gather, no deposit (FP32)
+  kPushSort = 2    // one that also sorts (SortOut)
 };
 template <typename R>
-constexpr int push_blocks_per_sm(int mode) { return sizeof(R) == 4 ? 3 : 2; }
+constexpr int push_blocks_per_sm() { return sizeof(R) == 4 ? 3 : 2; }
 template <typename R>
-constexpr int push_threads(int mode) {
-  return sizeof(R) == 4 ? (mode == kPushFree ? 512 : 384) : 256;
-}
+constexpr int push_threads() { return sizeof(R) == 4 ? 384 : 256; }
 // Slots that fill less than kPushFewWaves such waves are pushed by as many
 // warps in blocks of kPushFewThreads instead: the scheduler deals them out over
 // all SMs, where the large blocks of a partial wave fill some SMs and leave the
@@ -228,7 +225,7 @@ constexpr int push_threads(int mode) {
 // (74.6), 1.5e6 107.7 -> 105.9; FP64: 2e4 66.7 -> 52.8 (49.8), 1e5 157 -> 147
 // (145), 2e5 278 -> 252, 5e5 592 -> 562.  Beyond about eight waves the twelve
 // warps of a large block gain more from the L1 lines that they share: 1e7 655
-// (64 threads: 661), an unbounded 8e6 144 (150), FP64 1e6 level.
+// (64 threads: 661), FP64 1e6 level.
 constexpr int kPushFewThreads = 64, kPushFewWaves = 8;
 // resident 256-thread blocks per SM of the field and heating kernels (their
 // launch bounds); they are launched as one wave of sm_count times this many

@@ -26,14 +26,14 @@
 
 namespace hpic {
 
-// MODE: a plain step, one that also keys the next sort (ko), one that also
-// sorts (so says where the electrons go), or a plain one in an unbounded
-// medium; the other modes' code is compiled out.
+// MODE: a plain step, one that also keys the next sort (ko), or one that
+// also sorts (so says where the electrons go); the other modes' code is
+// compiled out.
 template <typename R, int NS, int MODE>
 // Launched as one persistent wave in the shape push_threads/push_blocks_per_sm
 // give, or with as many warps in smaller blocks (kPushFewThreads); FP32 gains
 // from the warps up to the register count at which spills begin.
-__global__ void __launch_bounds__(push_threads<R>(MODE), push_blocks_per_sm<R>(MODE))
+__global__ void __launch_bounds__(push_threads<R>(), push_blocks_per_sm<R>())
 k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__restrict__ tab,
        Counters *cnt, TallyView tv, const SortOut<R> so, const KeyOut<R> ko) {
   after_previous();
@@ -43,7 +43,7 @@ k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__rest
   if (threadIdx.x < kAccN) sums[threadIdx.x] = 0.0;
   __syncthreads();
   extern __shared__ __align__(16) unsigned char dyn[];  // the warps' deposit stages
-  R *stage = reinterpret_cast<R *>(dyn) + (threadIdx.x >> 5) * push_warp_words<R, MODE>();
+  R *stage = reinterpret_cast<R *>(dyn) + (threadIdx.x >> 5) * dep_words<R>();
   StepCtx sc;
   sc.step_ll = cnt->step;
   sc.step = (uint32_t)sc.step_ll;
@@ -58,13 +58,10 @@ k_push(const Consts K, const HotK<R> h, PView<R> p, GView<R> gv, const R *__rest
   // warp-uniform loop: every lane reaches the warp-cooperative deposits
   const int lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long first = blockIdx.x * (long long)blockDim.x + (threadIdx.x - lane);
-  if constexpr (reads_ahead<R, MODE>()) {
-    if (first < n) read_ahead(p, first, stage);
-  }
-  for (long long base = first; base < n; base += stride)
+  for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x - lane); base < n;
+       base += stride)
     push_warp<R, NS, MODE>(K, h, g, tab, tv, sc, p, base + lane, base + lane < n, acc, sums,
-                           stage, base + stride < n ? base + stride : -1, MODE == kPushSort ? &so : nullptr,
+                           stage, MODE == kPushSort ? &so : nullptr,
                            MODE == kPushSort ? &no_shift : nullptr,
                            MODE == kPushKeys ? &ko : nullptr);
 
@@ -222,9 +219,9 @@ __global__ void k_advance(const StepEnd end) {
 
 // ---------------------------------------------------------------- launchers
 
-template <typename R, int MODE>
-constexpr size_t push_stage_bytes(int threads = push_threads<R>(MODE)) {
-  return (threads / 32) * push_warp_words<R, MODE>() * sizeof(R);
+template <typename R>
+constexpr size_t push_stage_bytes(int threads = push_threads<R>()) {
+  return (threads / 32) * dep_words<R>() * sizeof(R);
 }
 
 cudaError_t prepare_push() {
@@ -233,18 +230,18 @@ cudaError_t prepare_push() {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  set((const void *)k_push<float, 1, kPushPlain>, push_stage_bytes<float, kPushPlain>());
-  set((const void *)k_push<float, 1, kPushKeys>, push_stage_bytes<float, kPushKeys>());
-  set((const void *)k_push<float, 1, kPushSort>, push_stage_bytes<float, kPushSort>());
-  set((const void *)k_push<float, 4, kPushPlain>, push_stage_bytes<float, kPushPlain>());
-  set((const void *)k_push<float, 4, kPushKeys>, push_stage_bytes<float, kPushKeys>());
-  set((const void *)k_push<float, 4, kPushSort>, push_stage_bytes<float, kPushSort>());
-  set((const void *)k_push<double, 1, kPushPlain>, push_stage_bytes<double, kPushPlain>());
-  set((const void *)k_push<double, 1, kPushKeys>, push_stage_bytes<double, kPushKeys>());
-  set((const void *)k_push<double, 1, kPushSort>, push_stage_bytes<double, kPushSort>());
-  set((const void *)k_push<double, 4, kPushPlain>, push_stage_bytes<double, kPushPlain>());
-  set((const void *)k_push<double, 4, kPushKeys>, push_stage_bytes<double, kPushKeys>());
-  set((const void *)k_push<double, 4, kPushSort>, push_stage_bytes<double, kPushSort>());
+  set((const void *)k_push<float, 1, kPushPlain>, push_stage_bytes<float>());
+  set((const void *)k_push<float, 1, kPushKeys>, push_stage_bytes<float>());
+  set((const void *)k_push<float, 1, kPushSort>, push_stage_bytes<float>());
+  set((const void *)k_push<float, 4, kPushPlain>, push_stage_bytes<float>());
+  set((const void *)k_push<float, 4, kPushKeys>, push_stage_bytes<float>());
+  set((const void *)k_push<float, 4, kPushSort>, push_stage_bytes<float>());
+  set((const void *)k_push<double, 1, kPushPlain>, push_stage_bytes<double>());
+  set((const void *)k_push<double, 1, kPushKeys>, push_stage_bytes<double>());
+  set((const void *)k_push<double, 1, kPushSort>, push_stage_bytes<double>());
+  set((const void *)k_push<double, 4, kPushPlain>, push_stage_bytes<double>());
+  set((const void *)k_push<double, 4, kPushKeys>, push_stage_bytes<double>());
+  set((const void *)k_push<double, 4, kPushSort>, push_stage_bytes<double>());
   return e;
 }
 
@@ -254,12 +251,12 @@ void launch_push_mode(const Consts &K, const HotK<R> &h, PView<R> p, GView<R> g,
                       const SortOut<R> &so, const KeyOut<R> &ko) {
   // one resident wave, or the blocks the slots fill (small ones where these are
   // few: kernels.h)
-  constexpr int full = push_threads<R>(MODE);
-  const long long warps = (long long)sm_count * push_blocks_per_sm<R>(MODE) * (full / 32);
+  constexpr int full = push_threads<R>();
+  const long long warps = (long long)sm_count * push_blocks_per_sm<R>() * (full / 32);
   const int threads = (cap + 31) / 32 < kPushFewWaves * warps ? kPushFewThreads : full;
   const long long want = (cap + threads - 1) / threads, wave = warps / (threads / 32);
   const int grid = (int)(want < wave ? want : wave);
-  const size_t smem = push_stage_bytes<R, MODE>(threads);
+  const size_t smem = push_stage_bytes<R>(threads);
   if (MODE == kPushSort)  // it follows the sort's scan
     launch_chained(k_push<R, NS, MODE>, grid, threads, smem, st, K, h, p, g, table, cnt, tv, so, ko);
   else
@@ -270,12 +267,6 @@ template <typename R, int NS>
 void launch_push_ns(const Consts &K, const HotK<R> &h, PView<R> p, GView<R> g, const R *table,
                     Counters *cnt, TallyView tv, long long cap, int sm_count, cudaStream_t st,
                     const SortOut<R> &so, const KeyOut<R> &ko) {
-  if constexpr (sizeof(R) == 4) {
-    if ((K.physics & P_UNBOUNDED) && !so.dst.x && !ko.keys) {
-      launch_push_mode<R, NS, kPushFree>(K, h, p, g, table, cnt, tv, cap, sm_count, st, so, ko);
-      return;
-    }
-  }
   if (so.dst.x)
     launch_push_mode<R, NS, kPushSort>(K, h, p, g, table, cnt, tv, cap, sm_count, st, so, ko);
   else if (ko.keys)

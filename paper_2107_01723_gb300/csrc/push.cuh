@@ -346,8 +346,7 @@ __device__ __noinline__ EmitOut<R> emit_photon(const EmitIn<R> e, StepCtx sc, ui
 // (the deposit's velocity factor), and its current is deposited.  NS: 1 for
 // a single-element solid (the element loops vanish), 4 for up to four
 // elements counted at run time.
-// FREE: an unbounded medium, known at compile time.
-template <typename R, int NS, bool FREE>
+template <typename R, int NS>
 __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const Grid<R> &g,
                                         const R *__restrict__ tab, const TallyView &tv,
                                         const StepCtx &sc, uint32_t id, R w, R &X, R &Y, R &Zc,
@@ -356,7 +355,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
   const int nx = h.nx, ny = h.ny, nz = h.nz;
 
   // ---- gather at x^n
-  const bool unbounded = FREE || (K.physics & P_UNBOUNDED) != 0;
+  const bool unbounded = (K.physics & P_UNBOUNDED) != 0;
   const Axis<R> ax = axis_weights(X, nx), ay = axis_weights(Y, ny), az = axis_weights(Zc, nz);
   R Ex = R(0), Ey = R(0), Ez = R(0), Bx = R(0), By = R(0), Bz = R(0);
   if (!unbounded) {
@@ -368,14 +367,13 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
     Bz = trilerp(g, 5, g.node(ax.iS, ay.iS, az.iN), ax.fS, ay.fS, az.fN);
   }
 
-  // Push, drag and scatter, in one of two forms.  FP64, and FP32 where there is
-  // no grid, hold the electron as direction and momentum, which saves roots,
-  // quotients and logarithms (FP64: 1e6 electrons 1670 -> 1290 us; FP32 in the
-  // unbounded medium 206 -> 195).  FP32 with the grid is held by the L1 data
-  // pipe and takes the same time either way (659 us at 1e7); it keeps the form
-  // whose every step is a rounded FP32 momentum, and with it the roundings of
-  // the runs already made.
-  constexpr bool kByDirection = sizeof(R) == 8 || FREE;
+  // Push, drag and scatter, in one of two forms.  FP64 holds the electron as
+  // direction and momentum, which saves roots, quotients and logarithms (1e6
+  // electrons 1670 -> 1290 us).  FP32 is held by the L1 data pipe with the grid
+  // (659 us at 1e7 either way) and by memory latency without it (2^23 electrons
+  // 206 against 195 us); it keeps the form whose every step is a rounded FP32
+  // momentum, and with it the roundings of the runs already made.
+  constexpr bool kByDirection = sizeof(R) == 8;
   R eps, gam = R(0), p = R(0), heat = 0;
   bool alive = true;
   if constexpr (kByDirection) {
@@ -833,47 +831,6 @@ __device__ __forceinline__ R ld_stream(const R *p) { return __ldcs(p); }
 template <typename R>
 __device__ __forceinline__ void st_stream(R *p, R v) { __stcs(p, v); }
 
-// Read-ahead of a warp's next 32 electrons: their x .. tau and ids, eight
-// 128-byte rows, go to shared memory by asynchronous 16-byte copies (two per
-// lane) while the warp works on the present ones.  Used in the unbounded
-// medium in FP32 (kPushFree), where DRAM latency took a third of the warps'
-// time and there is no deposit stage: 2^23 electrons 195 -> 154 us (2.6 ->
-// 3.3 TB/s; since the deviates' own work shrank 144 us, 3.5 TB/s), of which the
-// copies 10 us and the rest 48 warps per SM at 40 registers, for 36 at 56.
-// (With the grid on, it costs: the kernel is then held by the L1 data pipe,
-// 75 % busy, and the copies pass through it twice: 659 -> 690 us at 1e7.)
-template <typename R, int MODE>
-__host__ __device__ constexpr bool reads_ahead() { return sizeof(R) == 4 && MODE == kPushFree; }
-
-// shared-memory elements of a warp of the single-target kernel: its deposit
-// stage, or the electrons it reads ahead
-template <typename R, int MODE>
-__host__ __device__ constexpr int push_warp_words() {
-  return MODE == kPushFree ? 256 : dep_words<R>();
-}
-
-// slots [ip, ip + 32), ip a multiple of 32 (slot counts are multiples of 32,
-// so all 32 exist); buf: 256 words, 16-byte aligned
-template <typename R>
-__device__ __forceinline__ void read_ahead(const PView<R> &p, long long ip, R *buf) {
-  if constexpr (sizeof(R) == 4) {
-    const int lane = threadIdx.x & 31;
-    const long long stride = p.y - p.x;  // x .. tau, weight, id lie one stride apart
-    unsigned long long policy;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int c = lane + 32 * h, a = c >> 3;
-      const R *src = p.x + (a < 7 ? a : 8) * stride + ip + (c & 7) * 4;
-      const unsigned dst = (unsigned)__cvta_generic_to_shared(buf + c * 4);
-      asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst),
-                   "l"(src), "l"(policy)
-                   : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-}
-
 // The 32 lanes of a warp advance the electrons in slots ip (one per lane;
 // in_range false: nothing there) through the step, then deposit their
 // current and drag heat together through the warp's shared-memory stage
@@ -881,33 +838,20 @@ __device__ __forceinline__ void read_ahead(const PView<R> &p, long long ip, R *b
 // call it.  MODE kPushSort: the step also sorts, and *so (with *shift: see
 // SortOut; read only then, so it may stay in shared memory) says where the
 // electrons go; kPushKeys: the step also keys the next sort (*ko); the
-// pointers may be null otherwise.  Where reads_ahead: the stage holds the
-// electrons of ip or is getting them, and next is the first of the slots to
-// read into it once these are taken, or -1.
+// pointers may be null otherwise.
 template <typename R, int NS, int MODE>
 __device__ __forceinline__ void push_warp(const Consts &K, const HotK<R> &h, const Grid<R> &g,
                                           const R *__restrict__ tab, const TallyView &tv,
                                           const StepCtx &sc, const PView<R> &p, long long ip,
                                           bool in_range, Acc<R> &acc, double *rare,
-                                          R *__restrict__ stage, long long next,
-                                          const SortOut<R> *so,
+                                          R *__restrict__ stage, const SortOut<R> *so,
                                           const long long *shift, const KeyOut<R> *ko) {
   constexpr bool SORT = MODE == kPushSort;
   bool live = false, dep = false;
   uint32_t id = kDead;
   R X = 0, Y = 0, Zc = 0, ux = 0, uy = 0, uz = 0, tau = 0, heat = 0, w = h.w, ig = 0;
   int heat_cell = -1;
-  if constexpr (reads_ahead<R, MODE>()) {
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncwarp();
-    const int lane = threadIdx.x & 31;
-    X = stage[lane]; Y = stage[32 + lane]; Zc = stage[64 + lane];
-    ux = stage[96 + lane]; uy = stage[128 + lane]; uz = stage[160 + lane];
-    tau = stage[192 + lane];
-    id = __float_as_uint(stage[224 + lane]);
-    __syncwarp();
-    if (next >= 0) read_ahead(p, next, stage);
-  } else if (in_range) {
+  if (in_range) {
     // the state is loaded together with the id, not after testing it, so
     // that a slot costs one memory round trip (a dead slot's values are
     // read and left unused)
@@ -930,7 +874,7 @@ __device__ __forceinline__ void push_warp(const Consts &K, const HotK<R> &h, con
   }
   if (live) {
     ++acc.n_steps;
-    dep = advance<R, NS, MODE == kPushFree>(K, h, g, tab, tv, sc, id, w, X, Y, Zc, ux, uy, uz, tau, acc, rare, heat,
+    dep = advance<R, NS>(K, h, g, tab, tv, sc, id, w, X, Y, Zc, ux, uy, uz, tau, acc, rare, heat,
                          heat_cell, ig);
     if constexpr (SORT) {  // loaded here so that no register holds them through the step
       const long long q =
@@ -964,7 +908,7 @@ __device__ __forceinline__ void push_warp(const Consts &K, const HotK<R> &h, con
       p.id[ip] = kDead;
     }
   }
-  if (MODE != kPushFree && !(K.physics & P_UNBOUNDED))  // uniform over the warp
+  if (!(K.physics & P_UNBOUNDED))  // uniform over the warp
     warp_deposit(g, stage, dep, w, X, Y, Zc, ux, uy, uz, ig, heat, heat_cell);
 }
 
