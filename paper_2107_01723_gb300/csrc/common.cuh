@@ -12,6 +12,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "numerics.cuh"
+
 namespace hpic {
 
 constexpr uint32_t kDead = 0xFFFFFFFFu;  // id of an absorbed/escaped slot
@@ -175,131 +177,6 @@ __device__ __forceinline__ double m_fcos2pi(double u) { return cospi(2.0 * u); }
 __device__ __forceinline__ float m_floor(float x) { return floorf(x); }
 __device__ __forceinline__ double m_floor(double x) { return floor(x); }
 
-// ---------------------------------------------------------------- FP64 off the FP64 unit
-// GB300 completes two FP64 operations per clock and SM, conversions from and
-// to FP64 included, so a warp-wide one holds the SM's FP64 unit for 16 clocks
-// where an integer instruction takes a fraction of one.  Conversions of
-// positive numbers well inside FP32's range are therefore done on the bits.
-// in_range: a double in [2^-40, 2^60); zero, negative, infinite and NaN
-// values are not (callers take the plain expressions then).
-__device__ __forceinline__ bool in_range(double x) {
-  return (unsigned)(__double2hiint(x) - 0x3d700000) < 0x06400000u;
-}
-// (float)x of an in_range x: round to nearest, ties to even
-__device__ __forceinline__ float narrow(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned m = __funnelshift_l(lo, hi, 3) - 0xc0000000u;  // 29 bits cut, exponent rebiased
-  return __uint_as_float(m + (((lo << 3) | (m & 1u)) > 0x80000000u ? 1u : 0u));
-}
-// (double)x of a positive normal x
-__device__ __forceinline__ double widen(float x) {
-  const unsigned b = __float_as_uint(x);
-  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
-}
-// the smaller of two positive numbers, by their bits
-__device__ __forceinline__ double min_positive(double a, double b) {
-  return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
-}
-
-// FP64 reciprocals and roots for the per-electron arithmetic, of positive normal
-// numbers well inside FP32's range (others take the plain expressions): from the
-// FP32 estimate by one step of the series in the residual e (about 1e-7), to e^2:
-// three operations for 1/x, five for x^(-1/2), of a unit that completes two per
-// clock and SM.
-__device__ __forceinline__ bool fp32_range(double x) {  // [2^-100, 2^100)
-  return (unsigned)(__double2hiint(x) - 0x39b00000) < 0x0c800000u;
-}
-__device__ __forceinline__ double m_rcp(double x) {
-  if (!fp32_range(x)) return 1.0 / x;
-  const double y = widen(__fdividef(1.0f, narrow(x)));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ double m_rsqrt(double x) {
-  if (!fp32_range(x)) return rsqrt(x);
-  const double y = widen(rsqrtf(narrow(x)));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y, e * fma(0.375, e, 0.5), y);
-}
-__device__ __forceinline__ double m_rsqrt_near(double x) { return m_rsqrt(x); }
-__device__ __forceinline__ double m_sqrt_near(double x) { return x * m_rsqrt(x); }
-__device__ __forceinline__ double m_div_near(double n, double d) { return n * m_rcp(d); }
-// p = sqrt(x) and 1/p
-__device__ __forceinline__ void m_sqrt_both(double x, double &p, double &inv) {
-  inv = m_rsqrt(x);
-  p = x * inv;
-}
-
-// ---- tables of the FP64 push
-// Logarithms and the circle's functions cost 20 to 30 FP64 operations each in
-// full generality.  By Tang's table-driven methods (ACM TOMS 15(2), 1989, and
-// 16(4), 1990) the logarithm of a normal number takes ten, and sine and cosine
-// of a 23-bit deviate of the circle, whose sector and rest are exact integers,
-// thirteen.  All errors are of a few 1e-16 of 1.  With them, small-angle series
-// and deviates and range tests by the bits the FP64 push of 1e6 electrons went
-// from 1290 to 1062 us.
-struct Fp64Tables {
-  double c[256], l[256];    // c: a 24-bit reciprocal of 1 + (j + 1/2)/256; l = -ln c
-  double cs[256], sn[256];  // of the angle 2 pi (j + 1/2)/256
-  static constexpr double ln(double x) {  // x in [1/2, 1]
-    const double y = (x - 1.0) / (x + 1.0), y2 = y * y;
-    double s = 0.0;
-    for (int k = 41; k >= 1; k -= 2) s = s * y2 + 1.0 / k;
-    return 2.0 * y * s;
-  }
-  static constexpr double sine(double a) {  // |a| <= pi/4
-    double s = 0.0;
-    for (int k = 19; k >= 1; k -= 2) s = 1.0 - s * a * a / ((k + 1) * (k + 2));
-    return a * s;
-  }
-  static constexpr double cosine(double a) {
-    double s = 0.0;
-    for (int k = 20; k >= 0; k -= 2) s = 1.0 - s * a * a / ((k + 1) * (k + 2));
-    return s;
-  }
-  constexpr Fp64Tables() : c(), l(), cs(), sn() {
-    constexpr double pi = 3.14159265358979323846;
-    for (int j = 0; j < 256; ++j) {
-      c[j] = (double)(float)(512.0 / (512.0 + 2 * j + 1));
-      l[j] = -ln(c[j]);
-      const int q = j / 64, r = j % 64;  // quadrant, and 2 r + 1 512ths of the circle in it
-      const bool far = r >= 32;          // beyond pi/4: by the complement
-      const double a = (far ? 127 - 2 * r : 2 * r + 1) * pi / 256.0;
-      const double s = far ? cosine(a) : sine(a), o = far ? sine(a) : cosine(a);
-      cs[j] = q == 0 ? o : (q == 1 ? -s : (q == 2 ? -o : s));
-      sn[j] = q == 0 ? s : (q == 1 ? o : (q == 2 ? -s : -o));
-    }
-  }
-};
-static __device__ const Fp64Tables kFp64 = Fp64Tables();
-
-__device__ __forceinline__ double table_log(double x) {
-  const int hi = __double2hiint(x);
-  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // not positive and normal
-  const int j = (hi >> 12) & 255;
-  const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
-  const double k = __hiloint2double(0x43300000, ((hi >> 20) - 1023) ^ (int)0x80000000) -
-                   4503601774854144.0;  // by the bits of k + 2^52 + 2^31
-  const double r = fma(m, __ldg(kFp64.c + j), -1.0);  // |r| < 2^-9 + 2^-23
-  double q = fma(r, -1.0 / 6.0, 0.2);
-  q = fma(r, q, -0.25);
-  q = fma(r, q, 1.0 / 3.0);
-  q = fma(r, q, -0.5);
-  q = fma(r, q, 1.0);
-  return fma(r, q, fma(k, 0.693147180559945309417232, __ldg(kFp64.l + j)));
-}
-// cos (and sin) of 2 pi u, u = (m + 1/2) 2^-23 the deviate of x
-__device__ __forceinline__ void table_turn(uint32_t x, double &s, double &c) {
-  const uint32_t m = x >> 9;
-  const int j = (int)(m >> 15), f = 2 * (int)(m & 0x7fffu) - 32767;  // 2^-24ths from the middle
-  const double a = (double)f * (3.14159265358979323846 / 8388608.0), t = a * a;
-  const double sa = fma(a * t, fma(t, 1.0 / 120.0, -1.0 / 6.0), a);
-  const double ca = fma(t, fma(t, fma(t, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
-  const double cj = __ldg(kFp64.cs + j), sj = __ldg(kFp64.sn + j);
-  c = fma(cj, ca, -(sj * sa));
-  s = fma(sj, ca, cj * sa);
-}
-
 // the push's logarithms: of a deviate, and the quick one
 __device__ __forceinline__ double p_log(double x) { return table_log(x); }
 __device__ __forceinline__ float p_flog(float x) { return m_flog(x); }
@@ -309,31 +186,6 @@ __device__ __forceinline__ void p_turn(uint32_t x, double &s, double &c) { table
 __device__ __forceinline__ void p_cos_turn(uint32_t x, double &c) {
   double s;
   table_turn(x, s, c);
-}
-
-// sine and cosine of a deflection: by their series up to |x| = 1/2 (to x^15 and
-// x^16: below 1e-18), where nearly all are
-__device__ __forceinline__ void m_sincos_small(double x, double *s, double *c) {
-  if ((__double2hiint(x) & 0x7fffffff) < 0x3fe00000) {
-    const double t = x * x;
-    double p = fma(t, -1.0 / 1307674368000.0, 1.0 / 6227020800.0);
-    p = fma(t, p, -1.0 / 39916800.0);
-    p = fma(t, p, 1.0 / 362880.0);
-    p = fma(t, p, -1.0 / 5040.0);
-    p = fma(t, p, 1.0 / 120.0);
-    p = fma(t, p, -1.0 / 6.0);
-    *s = fma(x * t, p, x);
-    double q = fma(t, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
-    q = fma(t, q, 1.0 / 479001600.0);
-    q = fma(t, q, -1.0 / 3628800.0);
-    q = fma(t, q, 1.0 / 40320.0);
-    q = fma(t, q, -1.0 / 720.0);
-    q = fma(t, q, 1.0 / 24.0);
-    q = fma(t, q, -0.5);
-    *c = fma(t, q, 1.0);
-  } else {
-    sincos(x, s, c);
-  }
 }
 
 // Sort key of cell (i, j, k): 4x4x4 tiles in x-fastest tile order, cells
@@ -407,49 +259,6 @@ __device__ __forceinline__ bool all_finite(double a, double b, double c, double 
 }
 
 // ---------------------------------------------------------------- reductions
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// A sum of reals with the accuracy of an FP64 sum of them that keeps off the
-// FP64 unit where it can.  GB300 completes two FP64 operations per clock and
-// SM, so one warp-wide FP64 add holds that unit for 16 clocks: the tree sums
-// at the end of a kernel cost microseconds there.  An FP32 sum is carried as
-// a pair (hi, lo) by Knuth's branch-free two-sum (TAOCP vol. 2, 4.2.2), 48
-// bits wide, on the FP32 units.
-template <typename R>
-struct WideSum;
-template <>
-struct WideSum<float> {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(hi, x), t = __fadd_rn(s, -hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -t)), __fadd_rn(x, -t)));
-    hi = s;
-  }
-  __device__ __forceinline__ void over_warp() {  // the total, in every lane
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
-      add(h);
-      lo = __fadd_rn(lo, l);
-    }
-  }
-  // (an infinite or NaN sum is hi's; lo is NaN then)
-  __device__ __forceinline__ double value() const {
-    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
-  }
-};
-template <>
-struct WideSum<double> {
-  double v = 0.0;
-  __device__ __forceinline__ void add(double x) { v += x; }
-  __device__ __forceinline__ void over_warp() { v = warp_sum(v); }
-  __device__ __forceinline__ double value() const { return v; }
-};
-
 // warp-aggregated atomic increment: lanes with equal keys share one atomic
 __device__ __forceinline__ uint32_t agg_inc(uint32_t *ctr, uint32_t key) {
   const unsigned mask = __activemask();

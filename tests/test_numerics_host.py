@@ -1,0 +1,82 @@
+"""The push's own FP64 functions, built for the host with the hardware's estimates at
+their worst, against 60-digit values: each within the error that the library function
+it stands for is given, over the range that the push uses.
+
+Unit of the errors: the last place (ulp) of the exact result.  log of CUDA's library is
+given 1, sincospi 2, sqrt and division are rounded (1/2)."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+mp = pytest.importorskip("mpmath")
+mp.mp.dps = 60
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2107_01723_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("numerics") / "numerics.so")
+    subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-shared", "-fPIC", "-I", CSRC,
+                    "-o", so, os.path.join(HERE, "numerics_host.cpp")], check=True)
+    return C.CDLL(so)
+
+
+def call(fn, *arrays, outs=1):
+    n = len(arrays[0])
+    out = [np.empty(n) for _ in range(outs)]
+    fn(*[a.ctypes.data_as(C.c_void_p) for a in (*arrays, *out)], C.c_long(n))
+    return out[0] if outs == 1 else out
+
+
+def worst(got, exact, given):
+    """The largest error in ulp of the exact result, and where."""
+    e = [abs(mp.mpf(float(g)) - x) / mp.mpf(float(np.spacing(abs(float(x))))) for g, x in zip(got, exact)]
+    i = int(np.argmax([float(v) for v in e]))
+    return float(e[i]), given[i]
+
+
+def deviates(m):
+    return (np.asarray(m, np.uint64) << 9).astype(np.uint32)
+
+
+def test_log_of_a_deviate(lib):
+    """ln u of the 23-bit deviate, also just below 1, where it is small."""
+    rng = np.random.default_rng(1)
+    top = (1 << 23) - 1
+    m = np.unique(np.concatenate([np.arange(64), top - np.arange(64), top - (np.logspace(0, 6.8, 600)).astype(int),
+                                  rng.integers(0, top, 1500)]))
+    x = (m + 0.5) * 2.0**-23
+    e, at = worst(call(lib.run_log, x), [mp.log(mp.mpf(v)) for v in x], x)
+    assert e <= 1.0, (e, at)
+
+
+def test_log_of_any_number(lib):
+    rng = np.random.default_rng(2)
+    near = np.concatenate([1 + s * np.logspace(-15, -0.5, 400) for s in (1, -1)])
+    rows = (1 + (np.arange(512) + 0.5) / 512)  # the rows' ends
+    x = np.concatenate([near, rows, np.nextafter(rows, 0), 2.0**rng.uniform(-1000, 1000, 600),
+                        2.0**rng.uniform(-40, 40, 1500), [2.0**-1022, np.finfo(float).max, 1.0]])
+    exact = [mp.log(mp.mpf(v)) for v in x]
+    keep = [i for i, v in enumerate(exact) if v != 0]
+    got = call(lib.run_log, x)
+    assert got[x == 1.0] == 0
+    e, at = worst(got[keep], [exact[i] for i in keep], x[keep])
+    assert e <= 1.05, (e, at)  # 1/2 for the result, 1/2 for r in the rows next to 1
+
+
+def test_circle(lib):
+    """Sine and cosine of the deviate, also at the quarters, where one is small."""
+    rng = np.random.default_rng(3)
+    quarters = np.concatenate([q * (1 << 21) + np.concatenate([np.arange(-40, 40), s * np.logspace(0.1, 6, 150).astype(int)])
+                               for q in range(4) for s in (1, -1)])
+    m = np.unique(np.concatenate([quarters % (1 << 23), rng.integers(0, 1 << 23, 1500)]))
+    turn = [(mp.mpf(int(v)) + mp.mpf(1) / 2) / 2**23 for v in m]
+    s, c = call(lib.run_turn, deviates(m), outs=2)
+    for got, exact in ((s, [mp.sin(2 * mp.pi * t) for t in turn]), (c, [mp.cos(2 * mp.pi * t) for t in turn])):
+        e, at = worst(got, exact, m)
+        assert e <= 2.0, (e, at)
