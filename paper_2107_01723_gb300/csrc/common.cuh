@@ -202,11 +202,10 @@ __device__ __forceinline__ R kinetic(R ux, R uy, R uz) {
   return m_div_rn(u2, R(1) + m_sqrt_rn(R(1) + u2));
 }
 
-// the same of u^2, with gamma: near-rounded
-template <typename R>
-__device__ __forceinline__ R kinetic_near(R u2, R &gam) {
-  gam = m_sqrt_near(R(1) + u2);
-  return m_div_near(u2, R(1) + gam);
+// the same of u^2, with gamma, in FP64 off the FP64 unit's root and division
+__device__ __forceinline__ double kinetic_near(double u2, double &gam) {
+  gam = m_sqrt_near(1.0 + u2);
+  return m_div_near(u2, 1.0 + gam);
 }
 
 // momentum |u| of kinetic energy e (m_e c^2)
@@ -231,13 +230,13 @@ __device__ __forceinline__ void rotate(R &dx, R &dy, R &dz, R ct, R st, R cp, R 
 // The same rotation with the sums over the frame's vectors carried out: with
 // (qx, qy) = st (cp, sp), V = sg dx qx + dy qy and T = a V the rotated
 // direction is (dx (ct + T) + qx, dy (ct + T) + sg qy, dz ct - V).
-template <typename R>
-__device__ __forceinline__ void rotate_near(R &dx, R &dy, R &dz, R ct, R st, R cp, R sp) {
-  const bool up = dz >= R(0);
-  const R qx = st * cp, qy = st * sp;
-  const R V = (up ? dx : -dx) * qx + dy * qy;
-  const R T = m_div_near(V, (up ? R(-1) : R(1)) - dz);
-  const R k = ct + T;
+__device__ __forceinline__ void rotate_near(double &dx, double &dy, double &dz, double ct,
+                                            double st, double cp, double sp) {
+  const bool up = dz >= 0.0;
+  const double qx = st * cp, qy = st * sp;
+  const double V = (up ? dx : -dx) * qx + dy * qy;
+  const double T = V * m_rcp((up ? -1.0 : 1.0) - dz);
+  const double k = ct + T;
   dx = dx * k + qx;
   dy = dy * k + (up ? qy : -qy);
   dz = dz * ct - V;

@@ -393,8 +393,8 @@ k_live_energy(const Consts K, PView<R> p, const Counters *cnt, double *dst) {
     // (the shared weight comes in at the end; reading the
     // tallies at 1e7 electrons 0.57 -> 0.43 ms)
     const double ux = p.ux[ip], uy = p.uy[ip], uz = p.uz[ip];
-    const double u2 = ux * ux + uy * uy + uz * uz, g2 = 1.0 + u2;
-    const double k = u2 * m_rcp(1.0 + g2 * m_rsqrt(g2));
+    double gam;
+    const double k = kinetic_near(ux * ux + uy * uy + uz * uz, gam);
     e = K.weighted ? fma((double)p.w[ip], k, e) : e + k;
   }
   const double v[1] = {K.weighted ? e : e * K.w};

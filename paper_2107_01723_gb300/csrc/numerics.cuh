@@ -33,11 +33,13 @@ __device__ __forceinline__ double min_positive(double a, double b) {
   return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
 }
 
-// FP64 reciprocals and roots for the per-electron arithmetic, of positive normal
-// numbers well inside FP32's range (others take the plain expressions): from the
-// FP32 estimate by one step of the series in the residual e (about 1e-7), to e^2:
-// three operations for 1/x, five for x^(-1/2), of a unit that completes two per
-// clock and SM.
+// FP64 reciprocals, roots and quotients for the per-electron arithmetic, of positive
+// normal numbers well inside FP32's range (others take the plain expressions): from
+// the FP32 estimate by one step of the series in the residual e (about 1e-7), to e^2:
+// three operations for 1/x, six for x^(-1/2), whose residual is exact but for one
+// rounding as the square of 24 bits fits.  Roots and quotients end with a step on
+// their own residual, so that all are rounded but for rare last places (at most
+// 0.501 of one off), as the library's are.
 __device__ __forceinline__ bool fp32_range(double x) {  // [2^-100, 2^100)
   return (unsigned)(__double2hiint(x) - 0x39b00000) < 0x0c800000u;
 }
@@ -50,16 +52,24 @@ __device__ __forceinline__ double m_rcp(double x) {
 __device__ __forceinline__ double m_rsqrt(double x) {
   if (!fp32_range(x)) return rsqrt(x);
   const double y = widen(rsqrtf(narrow(x)));
-  const double e = fma(-x * y, y, 1.0);
+  const double e = fma(-x, y * y, 1.0);
   return fma(y, e * fma(0.375, e, 0.5), y);
 }
-__device__ __forceinline__ double m_rsqrt_near(double x) { return m_rsqrt(x); }
-__device__ __forceinline__ double m_sqrt_near(double x) { return x * m_rsqrt(x); }
-__device__ __forceinline__ double m_div_near(double n, double d) { return n * m_rcp(d); }
+// sqrt(x), inv its reciprocal; half of inv by its exponent
+__device__ __forceinline__ double root_of(double x, double inv) {
+  const double s = x * inv;
+  const double h = __hiloint2double(__double2hiint(inv) - 0x00100000, __double2loint(inv));
+  return fma(fma(-s, s, x), h, s);
+}
+__device__ __forceinline__ double m_sqrt_near(double x) { return root_of(x, m_rsqrt(x)); }
+__device__ __forceinline__ double m_div_near(double n, double d) {
+  const double y = m_rcp(d), q = n * y;
+  return fma(fma(-q, d, n), y, q);
+}
 // p = sqrt(x) and 1/p
 __device__ __forceinline__ void m_sqrt_both(double x, double &p, double &inv) {
   inv = m_rsqrt(x);
-  p = x * inv;
+  p = root_of(x, inv);
 }
 
 // ---- tables of the FP64 push

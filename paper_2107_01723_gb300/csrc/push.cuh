@@ -398,7 +398,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
     // drag changes p alone and the scatter d alone, and the energy eps, gamma =
     // 1 + eps and their reciprocals serve every term, so that no root or
     // quotient is formed twice.  (u is rebuilt as p d after the collisions.)
-    const R inv = m_rsqrt_near(u2);
+    const R inv = m_rsqrt(u2);
     R inv_p = inv;
     p = u2 * inv;
     R dx = ux * inv, dy = uy * inv, dz = uz * inv;

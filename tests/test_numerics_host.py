@@ -80,3 +80,23 @@ def test_circle(lib):
     for got, exact in ((s, [mp.sin(2 * mp.pi * t) for t in turn]), (c, [mp.cos(2 * mp.pi * t) for t in turn])):
         e, at = worst(got, exact, m)
         assert e <= 2.0, (e, at)
+
+
+@pytest.mark.parametrize("off", [-2, 0, 2])
+def test_quotients_and_roots(lib, off):
+    """Rounded but for rare last places: 1/2 and what three terms of the residual's
+    series leave at an estimate of two last places off (4e-7 cubed: below 1e-3)."""
+    rng = np.random.default_rng(4)
+    x = np.concatenate([2.0**rng.uniform(-30, 30, 1500), 1 + rng.uniform(0, 1e-6, 300), 1 + 2.0**rng.uniform(-40, 2, 300)])
+    y = np.concatenate([2.0**rng.uniform(-30, 30, 1800), rng.uniform(1, 2, 300)])
+    lib.set_off(off)
+    try:
+        X, Y = [mp.mpf(v) for v in x], [mp.mpf(v) for v in y]
+        for fn, given, exact in ((lib.run_rcp, (x,), [1 / v for v in X]),
+                                 (lib.run_rsqrt, (x,), [1 / mp.sqrt(v) for v in X]),
+                                 (lib.run_sqrt, (x,), [mp.sqrt(v) for v in X]),
+                                 (lib.run_div, (y, x), [b / a for a, b in zip(X, Y)])):
+            e, at = worst(call(fn, *given), exact, x)
+            assert e <= 0.501, (e, at)
+    finally:
+        lib.set_off(0)
