@@ -177,11 +177,10 @@ __device__ __forceinline__ R fsigma(const FieldCommon &K, double Ti) {
 }
 
 // ---------------------------------------------------------------- B, Eq. (A3), and heating
-// Faraday on the faces owned by node q, then heating of cell q; the cell's
-// Ohmic energy density (J/m^3) goes to `ohm`
+// Faraday on the faces owned by node q, then heating of cell q; returns the cell's
+// Ohmic energy density (J/m^3)
 template <typename R>
-__device__ __forceinline__ void bheat_node(const FieldK<R> &K, const GView<R> &g, unsigned node,
-                                           WideSum<R> &ohm) {
+__device__ __forceinline__ R bheat_node(const FieldK<R> &K, const GView<R> &g, unsigned node) {
   constexpr unsigned Z = sizeof(R), D = sizeof(double);
   const int nx = K.nx, ny = K.ny, nz = K.nz;
   const unsigned q = node * Z, sy = K.sy * Z, sz = K.sz * Z;
@@ -229,11 +228,10 @@ __device__ __forceinline__ void bheat_node(const FieldK<R> &K, const GView<R> &g
     // a cell without drag heat or current keeps T and eta (and adds no
     // Ohmic energy) unless e-i equilibration moves it
     const bool no_heat = (__double_as_longlong(Hc) << 1) == 0;  // +0 or -0
-    if (no_heat && jb2 == R(0) && !(K.physics & P_EI)) return;
+    if (no_heat && jb2 == R(0) && !(K.physics & P_EI)) return R(0);
     double Te = at<const double>(g.T, c * D);
     bool changed = false;
     const R ro = at<const R>(g.eta_r, c * Z) * K.F_ohm * jb2;
-    ohm.add(ro);
     R rho = ro;
     if (!no_heat) {
       const double h = Hc * K.F_H;
@@ -291,7 +289,9 @@ __device__ __forceinline__ void bheat_node(const FieldK<R> &K, const GView<R> &g
       at(g.eta, c * D) = e;
       if constexpr (sizeof(R) == 4) at(g.eta_r, c * Z) = in_range(e) ? narrow(e) : (float)e;
     }
+    return ro;
   }
+  return R(0);
 }
 
 }  // namespace hpic

@@ -22,19 +22,21 @@ __global__ void __launch_bounds__(256, kFieldBlocksPerSm) k_efield(const FieldK<
 template <typename R>
 __global__ void __launch_bounds__(256, kFieldBlocksPerSm)
 k_bheat(const FieldK<R> K, GView<R> g, TallyView tv, const StepEnd end) {
-  __shared__ double sum;
-  if (threadIdx.x == 0) sum = 0.0;
-  __syncthreads();
+  __shared__ WideSum<R> part[8];  // the warps' Ohmic sums
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   after_previous();
   // nothing in this kernel or after it in the step reads the counters
   if (end.cnt && blockIdx.x == 0 && threadIdx.x == 0) close_step(end);
-  WideSum<R> ohm;
+  WideSum<R> ohm{};
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < K.nvec; q += gridDim.x * blockDim.x)
-    bheat_node(K, g, q, ohm);
+    ohm.add(bheat_node(K, g, q));
   ohm.over_warp();
-  if ((threadIdx.x & 31) == 0 && ohm.value() != 0.0) atomicAdd(&sum, ohm.value());
+  if (lane == 0) part[warp] = ohm;
   __syncthreads();
-  if (threadIdx.x == 0 && sum != 0.0) atomicAdd(tv.tal + T_E_OHMIC, sum * K.dx3);
+  if (warp == 0) {
+    const double sum = warp_sum(lane < 8 ? part[lane].value() : 0.0);
+    if (lane == 0 && sum != 0.0) atomicAdd(tv.tal + T_E_OHMIC, sum * K.dx3);
+  }
 }
 
 // ---------------------------------------------------------------- batched field kernels
@@ -85,37 +87,46 @@ k_batch_efield(const BatchItem<R> *items, BatchDev d) {
   }
 }
 
-// (Each thread used to add its FP64 Ohmic sum to its target's shared double,
-// a compare-and-swap loop of up to 256 threads on one address.)
+// A warp meets each target for a few pieces only (three of 7.9e6 cells in 16
+// targets), so its sums over the lanes are many: they stay in FP32 parts, one of
+// each warp and target, and become FP64 at the kernel's end, 8 lanes to a target.
+// (16 targets: 133 us; with the sums made FP64 each time 171.  Each thread used to add
+// its FP64 sum to its target's shared double, a compare-and-swap loop of up to 256
+// threads on one address.)
 template <typename R>
 __global__ void __launch_bounds__(256, kBatchFieldBlocksPerSm)
 k_batch_bheat(const BatchItem<R> *items, BatchDev d) {
   extern __shared__ long long npref_s[];
   __shared__ FieldHot<R> hot[8];
-  double *ohm_s = reinterpret_cast<double *>(npref_s + d.n + 1);
+  WideSum<R> *part = reinterpret_cast<WideSum<R> *>(npref_s + d.n + 1);  // [n][8]
   after_previous();
   for (int t = threadIdx.x; t <= d.n; t += blockDim.x) npref_s[t] = d.npref[t];
-  for (int t = threadIdx.x; t < d.n; t += blockDim.x) ohm_s[t] = 0.0;
+  for (int t = threadIdx.x; t < 8 * d.n; t += blockDim.x) part[t] = WideSum<R>{};
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long N = npref_s[d.n];
   int t = -1;
-  WideSum<R> ohm;
-  auto flush = [&]() {  // the warp's sum to its target's
+  WideSum<R> ohm{};
+  auto flush = [&]() {
     ohm.over_warp();
-    if (lane == 0 && ohm.value() != 0.0) atomicAdd(ohm_s + t, ohm.value() * hot[warp].K.dx3);
-    ohm = WideSum<R>();
+    if (lane == 0) part[t * 8 + warp] = ohm;
+    ohm = WideSum<R>{};
   };
   for (long long w = blockIdx.x * 8ll + warp; w < N; w += gridDim.x * 8ll) {
     if (t >= 0 && npref_s[t + 1] <= w) flush();
     t = enter_target(hot[warp], items, npref_s, t, w);
     const unsigned q = (unsigned)(w - npref_s[t]) * 32u + lane;
-    if (q < hot[warp].K.nvec) bheat_node(hot[warp].K, hot[warp].g, q, ohm);
+    if (q < hot[warp].K.nvec) ohm.add(bheat_node(hot[warp].K, hot[warp].g, q));
   }
   if (t >= 0) flush();
   __syncthreads();
-  for (int u = threadIdx.x; u < d.n; u += blockDim.x)
-    if (ohm_s[u] != 0.0) atomicAdd(items[u].tv.tal + T_E_OHMIC, ohm_s[u]);
+  for (int u = threadIdx.x; u < (8 * d.n + 31) / 32 * 32; u += blockDim.x) {  // whole warps
+    double sum = u < 8 * d.n ? part[u].value() : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (u % 8 == 0 && sum != 0.0)
+      atomicAdd(items[u / 8].tv.tal + T_E_OHMIC, sum * items[u / 8].f.dx3);
+  }
 }
 
 // ---------------------------------------------------------------- counting sort
@@ -482,7 +493,7 @@ void launch_batch_efield(const BatchItem<R> *items, BatchDev d, int grid, cudaSt
 
 template <typename R>
 void launch_batch_bheat(const BatchItem<R> *items, BatchDev d, int grid, cudaStream_t st) {
-  const size_t sm = (d.n + 1) * sizeof(long long) + d.n * sizeof(double);
+  const size_t sm = (d.n + 1) * sizeof(long long) + 8 * d.n * sizeof(WideSum<R>);
   launch_chained(k_batch_bheat<R>, grid, 256, sm, st, items, d);
 }
 

@@ -244,38 +244,62 @@ __device__ __forceinline__ double warp_sum(double v) {
 // A sum of reals with the accuracy of an FP64 sum of them that keeps off the
 // FP64 unit where it can.  GB300 completes two FP64 operations per clock and
 // SM, so one warp-wide FP64 add holds that unit for 16 clocks: the tree sums
-// at the end of a kernel cost microseconds there.  An FP32 sum is carried as
-// a pair (hi, lo) by Knuth's branch-free two-sum (TAOCP vol. 2, 4.2.2), 48
-// bits wide, on the FP32 units.
+// at the end of a kernel cost microseconds there.  An FP32 sum is carried in
+// three parts by Knuth's branch-free two-sum (TAOCP vol. 2, 4.2.2), 72 bits
+// wide, on the FP32 units; what is rounded is the last part and, in value(),
+// the result.
 template <typename R>
 struct WideSum;
 template <>
 struct WideSum<float> {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = __fadd_rn(hi, x), t = __fadd_rn(s, -hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -t)), __fadd_rn(x, -t)));
-    hi = s;
+  float hi, mid, lo;  // all zero to begin with
+  // a + x in a, and what that rounding left
+  static __device__ __forceinline__ float into(float &a, float x) {
+    const float s = __fadd_rn(a, x), t = __fadd_rn(s, -a);
+    const float left = __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -t)), __fadd_rn(x, -t));
+    a = s;
+    return left;
   }
-  __device__ __forceinline__ void over_warp() {  // the total, in every lane
+  __device__ __forceinline__ void add(float x) {
+    lo = __fadd_rn(lo, into(mid, into(hi, x)));
+  }
+  __device__ __forceinline__ void over_lanes(int first) {  // of 2 first lanes, in every lane
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+    for (int o = first; o > 0; o >>= 1) {
+      const float h = __shfl_xor_sync(0xffffffffu, hi, o), m = __shfl_xor_sync(0xffffffffu, mid, o);
+      const float l = __shfl_xor_sync(0xffffffffu, lo, o);
       add(h);
-      lo = __fadd_rn(lo, l);
+      lo = __fadd_rn(__fadd_rn(lo, l), into(mid, m));
     }
   }
-  // (an infinite or NaN sum is hi's; lo is NaN then)
+  __device__ __forceinline__ void over_warp() { over_lanes(16); }  // the total, in every lane
+  // (an infinite or NaN sum is hi's; the other parts are NaN then)
   __device__ __forceinline__ double value() const {
-    return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+    return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
   }
 };
 template <>
 struct WideSum<double> {
-  double v = 0.0;
+  double v;
   __device__ __forceinline__ void add(double x) { v += x; }
-  __device__ __forceinline__ void over_warp() { v = warp_sum(v); }
+  __device__ __forceinline__ void over_lanes(int first) {
+#pragma unroll
+    for (int o = first; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
+  __device__ __forceinline__ void over_warp() { over_lanes(16); }
   __device__ __forceinline__ double value() const { return v; }
 };
+
+// The warp's sums of two values of each lane, of a in lanes 0 to 15 and of b in lanes
+// 16 to 31: a half each, after each half has sent the other its share.
+template <typename R>
+__device__ __forceinline__ WideSum<R> warp_sums(R a, R b) {
+  const bool upper = (threadIdx.x & 16) != 0;
+  WideSum<R> s{};
+  s.add(upper ? b : a);
+  s.add(__shfl_xor_sync(0xffffffffu, upper ? a : b, 16));
+  s.over_lanes(8);
+  return s;
+}
 
 }  // namespace hpic

@@ -185,18 +185,14 @@ template <typename R>
 struct Acc {
   R W = 0, drag = 0;
   int n_cut = 0, n_steps = 0;
-  // the warp's totals, added by lane 0 to the shared array `dst` of kAccN doubles
+  // the warp's totals, added by lanes 0 and 16 to the shared array `dst` of kAccN doubles
   __device__ __forceinline__ void flush_warp(double *dst) const {
     const int cut = __reduce_add_sync(0xffffffffu, n_cut);
     const int steps = __reduce_add_sync(0xffffffffu, n_steps);
-    WideSum<R> w, d;
-    w.add(W);
-    d.add(drag);
-    w.over_warp();
-    d.over_warp();
-    if ((threadIdx.x & 31) == 0) {
-      if (w.value() != 0.0) atomicAdd(dst + A_W, w.value());
-      if (d.value() != 0.0) atomicAdd(dst + A_DRAG, d.value());
+    const double sum = warp_sums(W, drag).value();
+    const int lane = threadIdx.x & 31;
+    if ((lane & 15) == 0 && sum != 0.0) atomicAdd(dst + (lane ? A_DRAG : A_W), sum);
+    if (lane == 0) {
       if (cut) atomicAdd(dst + A_N_CUT, (double)cut);
       if (steps) atomicAdd(dst + A_N_STEPS, (double)steps);
     }

@@ -40,10 +40,15 @@ inline double rsqrt(double x) { return 1.0 / std::sqrt(x); }
 template <typename T>
 T __ldg(const T *p) { return *p; }
 inline float __fadd_rn(float a, float b) { return a + b; }
-// a warp's exchange, of one lane: the lanes' values are handed over in `other`
+// a warp's exchange as one lane sees it: over_warp() runs all its rounds, and only
+// that of `round` finds another lane's parts, the rest zeros
 const float *other = nullptr;
-inline float __shfl_xor_sync(unsigned, float, int) { return *other++; }
+int round_of = 0;
+inline float __shfl_xor_sync(unsigned, float, int o) { return o == round_of ? *other++ : 0.0f; }
 inline double __shfl_xor_sync(unsigned, double v, int) { return v; }
+struct {
+  unsigned x;
+} threadIdx;
 using std::fma;
 using std::isfinite;
 }  // namespace
@@ -51,6 +56,17 @@ using std::isfinite;
 #include "numerics.cuh"
 
 using namespace hpic;
+
+namespace {
+template <int parts>
+void exchange(WideSum<float> &mine, const WideSum<float> &theirs, int o) {
+  float v[parts];
+  std::memcpy(v, &theirs, sizeof(v));
+  other = v;
+  round_of = o;
+  mine.over_warp();
+}
+}  // namespace
 
 extern "C" {
 void set_off(int n) { off = n; }
@@ -66,5 +82,19 @@ void run_rsqrt(const double *x, double *y, long n) { for (long i = 0; i < n; ++i
 void run_sqrt(const double *x, double *y, long n) { for (long i = 0; i < n; ++i) y[i] = m_sqrt_near(x[i]); }
 void run_div(const double *a, const double *b, double *y, long n) {
   for (long i = 0; i < n; ++i) y[i] = m_div_near(a[i], b[i]);
+}
+// `steps` values of each of 32 lanes, x[step][lane], then the sum over the warp by
+// exchanges: lane 0's total
+double warp_total(const float *x, long steps) {
+  WideSum<float> lane[32] = {};
+  for (long i = 0; i < steps; ++i)
+    for (int l = 0; l < 32; ++l) lane[l].add(x[32 * i + l]);
+  constexpr int parts = sizeof(WideSum<float>) / sizeof(float);
+  for (int o = 16; o > 0; o >>= 1) {
+    WideSum<float> before[32];
+    std::memcpy(before, lane, sizeof(lane));
+    for (int l = 0; l < 32; ++l) exchange<parts>(lane[l], before[l ^ o], o);
+  }
+  return lane[0].value();
 }
 }

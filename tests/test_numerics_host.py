@@ -100,3 +100,28 @@ def test_quotients_and_roots(lib, off):
             assert e <= 0.501, (e, at)
     finally:
         lib.set_off(0)
+
+
+@pytest.mark.parametrize("steps", [1, 3, 40])
+@pytest.mark.parametrize("kind", ["alike", "spread", "signs"])
+def test_warp_sums(lib, steps, kind):
+    """FP32 values summed by a warp as exactly as an FP64 sum of them: within one
+    rounding in FP64 of the exact sum, and of what the values' own size allows."""
+    import math
+    lib.warp_total.restype = C.c_double
+    rng = np.random.default_rng(steps)
+    for _ in range(200):
+        x = rng.uniform(0.5, 1, 32 * steps)
+        if kind != "alike":
+            x *= 2.0**rng.uniform(-24, 0, x.size)
+        if kind == "signs":
+            x *= rng.choice([-1, 1], x.size)
+        x = x.astype(np.float32)
+        exact = math.fsum(x.astype(float))
+        got = lib.warp_total(x.ctypes.data_as(C.c_void_p), C.c_long(steps))
+        # the result's rounding, and below that the last part's (24 bits, 48 below the largest)
+        bound = 2.0**-53 * abs(exact) + 2.0**-68 * float(np.sum(np.abs(x, dtype=float)))
+        assert abs(got - exact) <= bound, (got, exact, abs(got - exact) / bound)
+    inf = np.zeros(32, np.float32)
+    inf[3] = np.inf
+    assert lib.warp_total(inf.ctypes.data_as(C.c_void_p), C.c_long(1)) == np.inf
