@@ -608,12 +608,15 @@ T *device_array(T *p, long long n) {
 // ms for a grid of 33 MB (with the pages supplied, 0.2 in five of five, 10 in one
 // other; supplying them takes 1.7 ms, 0.14 where they are present).  The kernel
 // is asked for the pages: nothing is written here, and memory that it refuses, or
-// that is no pageable memory at all, is left for the copy to report.
+// that is no pageable memory at all, is left for the copy to report.  Small arrays
+// lie in pages that the allocator has kept: asking for them made a pass that reads
+// seven grids of 18 kB 1.69 -> 1.78 ms.
 void supply_pages(const void *p, size_t bytes) {
 #ifdef MADV_POPULATE_WRITE
+  if (bytes < (1u << 20)) return;
   cudaPointerAttributes a{};
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) cudaGetLastError();
-  else if (a.type == cudaMemoryTypeUnregistered && bytes) {
+  else if (a.type == cudaMemoryTypeUnregistered) {
     static const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
     const uintptr_t first = reinterpret_cast<uintptr_t>(p) / page * page;
     const uintptr_t end = reinterpret_cast<uintptr_t>(p) + bytes;
