@@ -154,26 +154,19 @@ inline __device__ __noinline__ double resistivity_any(double eta_hot, double eta
   return eta < eta_max ? eta : eta_max;
 }
 
-// F_sigma (App. B) of the ion temperature, for the FP32 push by an FP32
-// logarithm of the significand (below 0.35, error 3e-8) added in FP64 to the
-// exponent's: 5e-8 of the logarithm, times fs_q (below 1/4), which stays under
-// the rounding of the result
+// F_sigma (App. B) of the ion temperature; for the FP32 push within 2^-33 (times fs_q,
+// below 1/4) before it is rounded to FP32: the rounded value but for one in a thousand
 template <typename R>
 __device__ __forceinline__ R fsigma(const FieldCommon &K, double Ti) {
-  double half_log;
+  double log_Ti;
   if (sizeof(R) == 4 && in_range(Ti)) {
-    const unsigned b = __float_as_uint(narrow(Ti));
-    float m = __uint_as_float((b & 0x007fffffu) | 0x3f800000u);
-    int k = (int)(b >> 23) - 127;
-    if (m > 1.41421356f) {
-      m *= 0.5f;
-      ++k;
-    }
-    half_log = fma((double)k, 0.5 * 0.693147180559945309417232, 0.5 * (double)logf(m));
+    float rest;
+    log_parts(Ti, log_Ti, rest);
+    log_Ti += (double)rest;
   } else {
-    half_log = 0.5 * log(Ti);
+    log_Ti = table_log(Ti);
   }
-  return R(fma(K.fs_q, half_log + K.fs_c, 1.0));
+  return R(fma(K.fs_q, fma(0.5, log_Ti, K.fs_c), 1.0));
 }
 
 // ---------------------------------------------------------------- B, Eq. (A3), and heating

@@ -196,6 +196,29 @@ __device__ __forceinline__ double table_log(double x) {
   const double sum = base + r, left = r - (sum - base);  // |r| < |base|, or base is 0
   return sum + (left + fma(r2, q, rest));
 }
+// The same of a positive normal x for results kept in FP32: ln x = base + rest within
+// 2^-33, the short series and the last 29 bits of x in FP32 (two FP64 operations, and
+// what the sum takes)
+__device__ __forceinline__ void log_parts(double x, double &base, float &rest) {
+  const int xh = __double2hiint(x), up = xh + 0x800, j = (up >> 12) & 255;
+  const int mh = xh - (up & 0x7ff00000) + 0x3ff00000;  // of m
+  const int n = ((up + ((256 - Fp64Tables::kHalf) << 12)) >> 20) - 1023;
+  const double k = __hiloint2double(0x43300000, n ^ (int)0x80000000) - 4503601774854144.0;
+  const double2 *row = reinterpret_cast<const double2 *>(kFp64.log + j);
+  const double2 ch = __ldg(row);
+  const unsigned lo = (unsigned)__double2loint(x);
+  // m in 24 bits, cut, and what was cut; c, which has 24 bits, by its own bits
+  const float a = __uint_as_float(__funnelshift_l(lo, (unsigned)mh, 3) - 0xc0000000u);
+  const float b = (float)(lo & 0x1fffffffu) * (mh < 0x3ff00000 ? 0x1p-53f : 0x1p-52f);
+  const float c = __uint_as_float(
+      __funnelshift_l((unsigned)__double2loint(ch.x), (unsigned)__double2hiint(ch.x), 3) - 0xc0000000u);
+  const float p = __fmul_rn(a, c), r = __fadd_rn(p, -1.0f);  // exact, p being near 1
+  float q = fmaf(r, -0.25f, 1.0f / 3.0f);
+  q = fmaf(r, q, -0.5f);
+  const float s = fmaf(b, c, fmaf(a, c, -p));  // what r lacks: s/(1 + r) of the logarithm
+  rest = __fadd_rn(r, fmaf(__fmul_rn(r, r), q, fmaf(-s, r, s)));
+  base = fma(k, 0.693147180559945309417232, ch.y);  // (the rows' lo: below 2^-43)
+}
 // sine and cosine of 2 pi u, u = (n + 1/2) 2^-23 the deviate of x: 2 n + 1 2^-24ths
 // of the circle, f of them from the axis of row j
 __device__ __forceinline__ void table_turn(uint32_t x, double &s, double &c) {

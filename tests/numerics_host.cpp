@@ -40,6 +40,7 @@ inline double rsqrt(double x) { return 1.0 / std::sqrt(x); }
 template <typename T>
 T __ldg(const T *p) { return *p; }
 inline float __fadd_rn(float a, float b) { return a + b; }
+inline float __fmul_rn(float a, float b) { return a * b; }
 // a warp's exchange as one lane sees it: over_warp() runs all its rounds, and only
 // that of `round` finds another lane's parts, the rest zeros
 const float *other = nullptr;
@@ -71,6 +72,13 @@ void exchange(WideSum<float> &mine, const WideSum<float> &theirs, int o) {
 extern "C" {
 void set_off(int n) { off = n; }
 void run_log(const double *x, double *y, long n) { for (long i = 0; i < n; ++i) y[i] = table_log(x[i]); }
+void run_log_parts(const double *x, double *base, double *rest, long n) {
+  for (long i = 0; i < n; ++i) {
+    float r;
+    log_parts(x[i], base[i], r);
+    rest[i] = r;
+  }
+}
 void run_turn(const uint32_t *x, double *s, double *c, long n) {
   for (long i = 0; i < n; ++i) table_turn(x[i], s[i], c[i]);
 }

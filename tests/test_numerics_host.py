@@ -69,6 +69,17 @@ def test_log_of_any_number(lib):
     assert e <= 1.05, (e, at)  # 1/2 for the result, 1/2 for r in the rows next to 1
 
 
+def test_log_for_fp32_results(lib):
+    """In two parts, to 2^-33: of a temperature, and next to 1 and to the rows' ends."""
+    rng = np.random.default_rng(6)
+    rows = (1 + (np.arange(512) + 0.5) / 512)
+    x = np.concatenate([2.0**rng.uniform(-40, 60, 3000), rows, np.nextafter(rows, 0), np.nextafter(rows, 3),
+                        1 + np.logspace(-15, -1, 100), 1 - np.logspace(-15, -1, 100)])
+    base, rest = call(lib.run_log_parts, x, outs=2)
+    e = [float(abs(mp.mpf(float(b)) + mp.mpf(float(r)) - mp.log(mp.mpf(float(v))))) for b, r, v in zip(base, rest, x)]
+    assert max(e) <= 2.0**-33, (max(e) * 2.0**33, x[int(np.argmax(e))])
+
+
 def test_circle(lib):
     """Sine and cosine of the deviate, also at the quarters, where one is small."""
     rng = np.random.default_rng(3)
