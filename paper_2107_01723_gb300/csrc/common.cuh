@@ -227,21 +227,6 @@ __device__ __forceinline__ void rotate(R &dx, R &dy, R &dz, R ct, R st, R cp, R 
   dx = ox; dy = oy; dz = oz;
 }
 
-// The same rotation with the sums over the frame's vectors carried out: with
-// (qx, qy) = st (cp, sp), V = sg dx qx + dy qy and T = a V the rotated
-// direction is (dx (ct + T) + qx, dy (ct + T) + sg qy, dz ct - V).
-__device__ __forceinline__ void rotate_near(double &dx, double &dy, double &dz, double ct,
-                                            double st, double cp, double sp) {
-  const bool up = dz >= 0.0;
-  const double qx = st * cp, qy = st * sp;
-  const double V = (up ? dx : -dx) * qx + dy * qy;
-  const double T = V * m_rcp((up ? -1.0 : 1.0) - dz);
-  const double k = ct + T;
-  dx = dx * k + qx;
-  dy = dy * k + (up ? qy : -qy);
-  dz = dz * ct - V;
-}
-
 // none of them infinite or NaN: zero times each is zero (in FP64 by the
 // exponents, off the FP64 unit)
 __device__ __forceinline__ bool all_finite(float a, float b, float c, float d, float e, float f,

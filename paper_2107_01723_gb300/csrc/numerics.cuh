@@ -258,6 +258,24 @@ __device__ __forceinline__ void m_sincos_small(double x, double *s, double *c) {
   }
 }
 
+// Rotate unit d by polar angle (cos ct, sin st) at azimuth (cp, sp) in the frame of
+// Duff et al. (rotate() of common.cuh), with the sums over the frame's vectors carried
+// out: with (qx, qy) = st (cp, sp), sg = +1 for dz >= 0 and else -1, V = sg dx qx + dy qy
+// and T = -sg V/(1 + |dz|) the rotated direction is (dx (ct + T) + qx, dy (ct + T) +
+// sg qy, dz ct - V).  The divisor lies in [1, 2] for both signs of dz, where the quick
+// reciprocal serves every lane.
+__device__ __forceinline__ void rotate_near(double &dx, double &dy, double &dz, double ct,
+                                            double st, double cp, double sp) {
+  const bool up = dz >= 0.0;
+  const double qx = st * cp, qy = st * sp;
+  const double V = (up ? dx : -dx) * qx + dy * qy;
+  const double T = (up ? -V : V) * m_rcp(1.0 + fabs(dz));
+  const double k = ct + T;
+  dx = dx * k + qx;
+  dy = dy * k + (up ? qy : -qy);
+  dz = dz * ct - V;
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

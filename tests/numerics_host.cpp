@@ -51,6 +51,7 @@ struct {
   unsigned x;
 } threadIdx;
 using std::fma;
+using std::fabs;
 using std::isfinite;
 }  // namespace
 
@@ -84,6 +85,9 @@ void run_turn(const uint32_t *x, double *s, double *c, long n) {
 }
 void run_sincos(const double *x, double *s, double *c, long n) {
   for (long i = 0; i < n; ++i) m_sincos_small(x[i], s + i, c + i);
+}
+void run_rotate(double *d, const double *ct, const double *st, const double *cp, const double *sp, long n) {
+  for (long i = 0; i < n; ++i) rotate_near(d[3 * i], d[3 * i + 1], d[3 * i + 2], ct[i], st[i], cp[i], sp[i]);
 }
 void run_rcp(const double *x, double *y, long n) { for (long i = 0; i < n; ++i) y[i] = m_rcp(x[i]); }
 void run_rsqrt(const double *x, double *y, long n) { for (long i = 0; i < n; ++i) y[i] = m_rsqrt(x[i]); }

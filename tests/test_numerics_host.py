@@ -136,3 +136,28 @@ def test_warp_sums(lib, steps, kind):
     inf = np.zeros(32, np.float32)
     inf[3] = np.inf
     assert lib.warp_total(inf.ctypes.data_as(C.c_void_p), C.c_long(1)) == np.inf
+
+
+def test_rotation(lib):
+    """Against the frame's vectors summed out in long doubles, on both hemispheres, at
+    the poles and at the equator: some ten roundings of numbers below 2."""
+    L = np.longdouble
+    rng = np.random.default_rng(8)
+    n = 4000
+    d = rng.normal(size=(n, 3))
+    d[:200, :2] *= 1e-9
+    d[200:400, 2] *= 1e-17
+    d /= np.linalg.norm(d, axis=1)[:, None]
+    d[:4] = [[0, 0, 1], [0, 0, -1], [1, 0, 0], [0, 1, -0.0]]
+    theta, phi = rng.normal(size=n) * 0.3, rng.uniform(0, 2 * np.pi, n)
+    ct, st, cp, sp = np.cos(theta), np.sin(theta), np.cos(phi), np.sin(phi)
+    x, y, z = d.T.astype(L)
+    sg = np.where(z >= 0, L(1), L(-1))
+    a = -1 / (sg + z)
+    b = x * y * a
+    e1 = np.stack([1 + sg * x * x * a, sg * b, -sg * x])
+    e2 = np.stack([b, sg + y * y * a, -y])
+    want = d.T.astype(L) * ct + (e1 * cp + e2 * sp) * st.astype(L)
+    got = np.ascontiguousarray(d)
+    lib.run_rotate(*[v.ctypes.data_as(C.c_void_p) for v in (got, ct, st, cp, sp)], C.c_long(n))
+    assert float(np.max(np.abs(got.T - want))) <= 10 * 2.0**-52
