@@ -16,16 +16,20 @@ struct Axis {
 
 // The cell of X and the offset in it, by the bits of X + 2^(p-1), p the
 // significand's length, added rounding down: no conversion instruction (a
-// quarter-rate unit in FP32, the FP64 unit in FP64).
+// quarter-rate unit in FP32, the FP64 unit in FP64).  Beyond the numbers whose cell
+// the bits hold, far outside any box, it is a cell on that side: FP32 -1 and 2^23 and
+// more, FP64 -1 and 2^31 - 1.
 __device__ __forceinline__ int cell_of(float X, float &f) {
   const float t = __fadd_rd(X, 8388608.0f);
   f = X - (t - 8388608.0f);
-  return __float_as_int(t) - 0x4b000000;
+  return max(__float_as_int(t), 0x4affffff) - 0x4b000000;
 }
 __device__ __forceinline__ int cell_of(double X, double &f) {
   const double t = __dadd_rd(X, 4503599627370496.0);
   f = X - (t - 4503599627370496.0);
-  return __double2loint(t);
+  const int hi = __double2hiint(t), lo = __double2loint(t);
+  if (hi == 0x43300000 && lo >= 0) return lo;
+  return hi < 0x43300000 ? -1 : 0x7fffffff;
 }
 
 // Linear weights along one axis; X in cells, in [0, n].  The half-staggered
