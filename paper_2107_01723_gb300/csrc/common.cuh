@@ -139,9 +139,9 @@ __device__ __forceinline__ double unif<double>(uint32_t x) {  // 1 + m 2^-23 by 
 __device__ __forceinline__ float m_log(float x) { return logf(x); }
 __device__ __forceinline__ double m_log(double x) { return log(x); }
 // hardware log (absolute error ~5e-7) for terms of order 1-10 whose error
-// budget allows it; exact log in double precision
+// budget allows it; the table-driven one in double precision
 __device__ __forceinline__ float m_flog(float x) { return __logf(x); }
-__device__ __forceinline__ double m_flog(double x) { return log(x); }
+__device__ __forceinline__ double m_flog(double x) { return table_log(x); }
 __device__ __forceinline__ float m_exp(float x) { return expf(x); }
 __device__ __forceinline__ double m_exp(double x) { return exp(x); }
 __device__ __forceinline__ float m_expm1(float x) { return expm1f(x); }
@@ -160,33 +160,21 @@ __device__ __forceinline__ void m_sincos2pi(double u, double *s, double *c) { si
 // IEEE rounding where the push converts between an electron's energy and
 // its momentum (kinetic, u_of_eps, the rescale after drag or a photon) and
 // where it builds the frame of a rotation, so that no systematic rounding
-// bias enters an energy change that no tally records.
+// bias enters an energy change that no tally records.  (The FP64 push has its
+// own, rounded but for rare last places: numerics.cuh.)
 __device__ __forceinline__ float m_sqrt_rn(float x) { return __fsqrt_rn(x); }
 __device__ __forceinline__ double m_sqrt_rn(double x) { return sqrt(x); }
 __device__ __forceinline__ float m_div_rn(float a, float b) { return __fdiv_rn(a, b); }
 __device__ __forceinline__ double m_div_rn(double a, double b) { return a / b; }
 __device__ __forceinline__ float m_rsqrt_rn(float x) { return __frsqrt_rn(x); }
-__device__ __forceinline__ double m_rsqrt_rn(double x) { return 1.0 / sqrt(x); }
-// cos(2 pi u) for u in (0, 1): in FP32 from the hardware unit on the angle
+// cos(2 pi u) for u in (0, 1) in FP32: from the hardware unit on the angle
 // 2 pi (u - 1) for u > 1/2 (exact shift, |angle| <= pi, absolute error
-// about 5e-7); exact cospi in FP64
+// about 5e-7)
 __device__ __forceinline__ float m_fcos2pi(float u) {
   return __cosf(6.28318530717958647692f * (u > 0.5f ? u - 1.0f : u));
 }
-__device__ __forceinline__ double m_fcos2pi(double u) { return cospi(2.0 * u); }
 __device__ __forceinline__ float m_floor(float x) { return floorf(x); }
 __device__ __forceinline__ double m_floor(double x) { return floor(x); }
-
-// the push's logarithms: of a deviate, and the quick one
-__device__ __forceinline__ double p_log(double x) { return table_log(x); }
-__device__ __forceinline__ float p_flog(float x) { return m_flog(x); }
-__device__ __forceinline__ double p_flog(double x) { return table_log(x); }
-// sine and cosine of the deviate x of the circle; its cosine for a normal deviate
-__device__ __forceinline__ void p_turn(uint32_t x, double &s, double &c) { table_turn(x, s, c); }
-__device__ __forceinline__ void p_cos_turn(uint32_t x, double &c) {
-  double s;
-  table_turn(x, s, c);
-}
 
 // Sort key of cell (i, j, k): 4x4x4 tiles in x-fastest tile order, cells
 // x-fastest inside a tile, so consecutive electrons share a compact box.
@@ -202,7 +190,7 @@ __device__ __forceinline__ R kinetic(R ux, R uy, R uz) {
   return m_div_rn(u2, R(1) + m_sqrt_rn(R(1) + u2));
 }
 
-// the same of u^2, with gamma, in FP64 off the FP64 unit's root and division
+// the same of u^2, with gamma, for the FP64 push
 __device__ __forceinline__ double kinetic_near(double u2, double &gam) {
   gam = m_sqrt_near(1.0 + u2);
   return m_div_near(u2, 1.0 + gam);

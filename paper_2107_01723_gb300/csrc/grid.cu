@@ -8,8 +8,6 @@
 //   k_table  : inverse-CDF bremsstrahlung table from the closed-form CDF
 #include "fields.cuh"
 
-#include <type_traits>
-
 namespace hpic {
 
 template <typename R>

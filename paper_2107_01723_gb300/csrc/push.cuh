@@ -131,7 +131,7 @@ __device__ __forceinline__ R trilerp(const Grid<R> &g, int c, int b, R fx, R fy,
 // G(u0) = integral_{u0}^{1} s(u)/u du for s(u) = (4/3)(1-u) + u^2
 template <typename R>
 __device__ __forceinline__ R shape_G(R u0) {
-  return R(4.0 / 3.0) * (-p_flog(u0) - (R(1) - u0)) + R(0.5) * (R(1) - u0 * u0);
+  return R(4.0 / 3.0) * (-m_flog(u0) - (R(1) - u0)) + R(0.5) * (R(1) - u0 * u0);
 }
 
 // Photon energy from the inverse-CDF table (rows: ln eps, columns: the
@@ -410,7 +410,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
     } else if (K.physics & P_DRAG) {
       const R ig = m_rcp(gam);
       // ln(eps) + ln(gamma + 1)/2, and the bracket's terms in 1/gamma
-      const R br0 = R(0.5) * p_flog(eps * eps * (gam + R(1))) +
+      const R br0 = R(0.5) * m_flog(eps * eps * (gam + R(1))) +
                     ((R(0.909) * ig - R(0.818)) * ig - R(0.246));
       const R inv_beta = gam * inv;
       R de = R(0);
@@ -440,18 +440,18 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
 #pragma unroll
       for (int s = 0; s < NS; ++s) {  // the elements' variances add
         if (NS > 1 && s >= h.n_solids) break;
-        R lg = p_flog(h.K_lg[s] * p);
+        R lg = m_flog(h.K_lg[s] * p);
         lg = lg < R(0) ? R(0) : lg;
         var += h.K_sc[s] * lg;
       }
       var *= gam * inv_p * (inv_p * inv_p);
       R s2, c2, st, ct;
       // Box-Muller normal deviate (its cosine changes only the deflection)
-      R normal;
-      p_cos_turn(r0.b, normal);
-      const R theta = m_sqrt(var * (R(-2) * p_log(unif<R>(r0.a)))) * normal;
+      R normal, unused;
+      table_turn(r0.b, unused, normal);
+      const R theta = m_sqrt(var * (R(-2) * table_log(unif<R>(r0.a)))) * normal;
       m_sincos_small(theta, &st, &ct);
-      p_turn(r0.c, s2, c2);
+      table_turn(r0.c, s2, c2);
       rotate_near(dx, dy, dz, ct, st, c2, s2);
     }
     if (K.physics & (P_DRAG | P_SCATTER)) {
