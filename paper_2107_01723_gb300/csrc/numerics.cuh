@@ -62,9 +62,13 @@ __device__ __forceinline__ double root_of(double x, double inv) {
   return fma(fma(-s, s, x), h, s);
 }
 __device__ __forceinline__ double m_sqrt_near(double x) { return root_of(x, m_rsqrt(x)); }
+// n/d, inv the reciprocal of d
+__device__ __forceinline__ double quotient_of(double n, double d, double inv) {
+  const double q = n * inv;
+  return fma(fma(-q, d, n), inv, q);
+}
 __device__ __forceinline__ double m_div_near(double n, double d) {
-  const double y = m_rcp(d), q = n * y;
-  return fma(fma(-q, d, n), y, q);
+  return quotient_of(n, d, m_rcp(d));
 }
 // p = sqrt(x) and 1/p
 __device__ __forceinline__ void m_sqrt_both(double x, double &p, double &inv) {

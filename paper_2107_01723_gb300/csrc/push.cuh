@@ -429,7 +429,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
         heat += w * de;
         eps = eps1;
         gam = R(1) + eps;
-        m_sqrt_both(eps * (gam + R(1)), p, inv_p);
+        m_sqrt_both(eps * (eps + R(2)), p, inv_p);
       }
     }
 
@@ -537,7 +537,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
     R dtau;
     if constexpr (kByDirection) {
       const R inv_eps = m_rcp(eps);
-      dtau = h.K_tau * (p * inv_eps) * shape_G(h.k_min * inv_eps);
+      dtau = quotient_of(h.K_tau * p, eps, inv_eps) * shape_G(quotient_of(h.k_min, eps, inv_eps));
     } else {
       dtau = h.K_tau * u_of_eps(eps) / eps * shape_G(h.k_min / eps);
     }
@@ -558,7 +558,6 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
       if (o.xa != 0.0) atomicAdd(rare + A_XA, o.xa);
       atomicAdd(rare + A_N_EMIT, 1.0);
       tau = o.tau;
-      gam = R(1) + o.eps;
       ux = o.ux; uy = o.uy; uz = o.uz;
       heat += o.heat;
       alive = o.alive;
@@ -574,8 +573,14 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
   }
 
   // ---- move, then escape or reflux at each face crossed (out of line: rare)
-  if constexpr (kByDirection) ig = m_rcp(gam);
-  else ig = R(1) / m_sqrt(R(1) + ux * ux + uy * uy + uz * uz);
+  // (1/gamma of the momentum as it is stored: that of the energy leaves the rounding of
+  // |u| in the velocity)
+  auto inverse_gamma = [&]() {
+    const R g2 = R(1) + ux * ux + uy * uy + uz * uz;
+    if constexpr (kByDirection) return m_rsqrt(g2);
+    else return R(1) / m_sqrt(g2);
+  };
+  ig = inverse_gamma();
   R pos[3] = {X + ux * ig * h.cdt, Y + uy * ig * h.cdt, Zc + uz * ig * h.cdt};
   if (!unbounded && !(pos[0] >= R(0) && pos[0] <= R(nx) && pos[1] >= R(0) && pos[1] <= R(ny) &&
                       pos[2] >= R(0) && pos[2] <= R(nz))) {
@@ -590,8 +595,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
     if (!c.alive) return false;
     pos[0] = c.pos[0]; pos[1] = c.pos[1]; pos[2] = c.pos[2];
     ux = c.u[0]; uy = c.u[1]; uz = c.u[2];
-    if constexpr (kByDirection) ig = m_rsqrt(R(1) + ux * ux + uy * uy + uz * uz);
-    else ig = R(1) / m_sqrt(R(1) + ux * ux + uy * uy + uz * uz);
+    ig = inverse_gamma();
   }
   X = pos[0]; Y = pos[1]; Zc = pos[2];
 
