@@ -59,7 +59,7 @@ NCU_BATCH_CAPTURE_BLOCKS = 4
 # FP64 FLOP per particle-step of the FP64 k_push (2 per DFMA, 1 per DADD and
 # DMUL; ncu thread-level counts on config 1 in FP64, launches at steps 110
 # and 111) and the FP64 rate the GB300 is stated to have (TFLOP/s)
-NCU_FP64_FLOP_PER_PSTEP = 737.5
+NCU_FP64_FLOP_PER_PSTEP = 798.5
 FP64_STATED_TFLOPS = 1.25
 # the accuracy window: the injection (200 steps) and 1 ps beyond
 ACCURACY_STEPS = 2200

@@ -451,8 +451,8 @@ const char *hpic_batch_last_error(const hpic_batch *b);
 
 /* ------------------------------------------------------------------------
  * The paper's three-macro-electron estimate of the loss channels (Sec. III.B),
- * evaluated for many parameter sets at once, one GPU thread each (the
- * background heatmap of eta_e->gamma over intensity and Z).  Per set: a0
+ * evaluated for many parameter sets at once, three GPU threads each, one for
+ * every macro-electron (the background heatmap of eta_e->gamma over intensity and Z).  Per set: a0
  * from Eq. (1), mean energy <eps> = a0 m_e c^2 <sqrt(fg)>, injected count
  * N_e = I0 <fg> (pi r_fwhm^2/4)(t_fwhm sqrt(ln10/ln2)) eta_l2e / <eps>; the
  * exponential spectrum is cut at eps_th and eps_esc = kappa_esc a0 m_e c^2

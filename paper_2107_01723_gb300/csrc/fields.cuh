@@ -135,7 +135,7 @@ __device__ __forceinline__ R heat_increment(const FieldK<R> &K, R T, R rho) {
 // A heated cell took 29 FP64 instructions, the SM's FP64 unit a warp-wide one
 // in 19 clocks: 128 us for 128^3 cells, now 8 to 9 and 51 us; a batch of 7.9e6
 // cells (each target's constants in shared memory, its Ohmic sums made in the
-// warp) 542 -> 145 us.
+// warp) 542 -> 133 us.
 __device__ __forceinline__ double resistivity(const FieldCommon &K, double T, float Tf) {
   if (Tf > K.eta_Tlo && Tf < K.eta_Thi) return K.eta_max;
   double eta = times_pow_m32(K.eta_hot, T);
@@ -247,7 +247,7 @@ __device__ __forceinline__ R bheat_node(const FieldK<R> &K, const GView<R> &g, u
     if (K.physics & P_EI) {
       double Ti = at<const double>(g.Ti, c * D);
       const double d = Te - Ti, X = Te * K.ei_mi + Ti * K.ei_me;
-      // (1.4e5 aluminium cells with this and F_sigma: 60.7 -> 17.5 us by the
+      // (1.4e5 aluminium cells with this and F_sigma: 60.7 -> 16.2 us by the
       // power, the series and fsigma() in place of pow, expm1, a division and log)
       const double a = in_range(X) ? times_pow_m32(K.ei_a, X) : K.ei_a / pow(X, 1.5);
       const double b = K.Zstar * a, s = a + b;

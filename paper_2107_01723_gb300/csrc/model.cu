@@ -1,5 +1,5 @@
 // The paper's three-macro-electron estimate of the hot-electron loss
-// channels (arXiv 2107.01723, Sec. III.B), one GPU thread per parameter set.
+// channels (arXiv 2107.01723, Sec. III.B), one GPU thread per macro-electron.
 //
 // Per set: the exponential injection spectrum is cut at the X-ray threshold
 // and the escape energy into three macro-electrons (warm, emitting,
@@ -247,9 +247,9 @@ constexpr int kModelSets = 42;
 // shared memory.
 // One lane for a whole set, 128 sets to a block, left 46 of 152 SMs with work
 // for 5888 sets and the chain of three macro-electrons in every lane: 53.6 ms
-// for 64 intensities x 92 elements, now 9.4 ms (14.5 ms with the split alone,
-// before the FP64 operations of a step went from 262 to 165); about 47 ms for
-// any smaller number of sets, now 8.2 to 9.2 ms: the chain of one
+// for 64 intensities x 92 elements, now 9.4 ms (14.5 ms with the split alone;
+// the rest by 158 instead of 555 executed FP64 instructions per RK4 step); about
+// 47 ms for any smaller number of sets, now 8.2 to 9.2 ms: the chain of one
 // macro-electron's 1e3 steps.
 __global__ void __launch_bounds__(128) k_model(long long n, int per,
                                                const hpic_model_in *__restrict__ in,

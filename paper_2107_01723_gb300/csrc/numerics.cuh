@@ -86,7 +86,10 @@ __device__ __forceinline__ void m_sqrt_both(double x, double &p, double &inv) {
 // so that the errors are in proportion to the result, however small that is:
 // in its last places the logarithm of a deviate is 0.50 off at most (the library's
 // 0.53), of numbers near 1 0.70 (0.50), 0.25 on average like the library's; sine
-// and cosine 1.41 (sincospi 1.43), 0.25 on average (0.30).
+// and cosine 1.41 (sincospi 1.43), 0.25 on average (0.30).  (The FP64 push of 1e6
+// electrons takes 1150 us with them; with the library's logarithm and circle functions
+// it took 1290 although its roots and quotients were rougher.)
+//
 // Pairs of doubles for the tables, worked out by the compiler: sums and products
 // by Knuth's and Dekker's error-free forms (Dekker, "A floating-point technique
 // for extending the available precision", Numer. Math. 18, 1971).

@@ -369,7 +369,7 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
 
   // Push, drag and scatter, in one of two forms.  FP64 holds the electron as
   // direction and momentum, which saves roots, quotients and logarithms (1e6
-  // electrons 1670 -> 1290 us).  FP32 is held by the L1 data pipe with the grid
+  // electrons 1670 -> 1290 us; 1150 with the functions of numerics.cuh).  FP32 is held by the L1 data pipe with the grid
   // (659 us at 1e7 either way) and by memory latency without it (2^23 electrons
   // 206 against 195 us); it keeps the form whose every step is a rounded FP32
   // momentum, and with it the roundings of the runs already made.
