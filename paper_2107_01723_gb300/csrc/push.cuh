@@ -575,12 +575,8 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
   // ---- move, then escape or reflux at each face crossed (out of line: rare)
   // (1/gamma of the momentum as it is stored: that of the energy leaves the rounding of
   // |u| in the velocity)
-  auto inverse_gamma = [&]() {
-    const R g2 = R(1) + ux * ux + uy * uy + uz * uz;
-    if constexpr (kByDirection) return m_rsqrt(g2);
-    else return R(1) / m_sqrt(g2);
-  };
-  ig = inverse_gamma();
+  if constexpr (kByDirection) ig = m_rsqrt(R(1) + ux * ux + uy * uy + uz * uz);
+  else ig = R(1) / m_sqrt(R(1) + ux * ux + uy * uy + uz * uz);
   R pos[3] = {X + ux * ig * h.cdt, Y + uy * ig * h.cdt, Zc + uz * ig * h.cdt};
   if (!unbounded && !(pos[0] >= R(0) && pos[0] <= R(nx) && pos[1] >= R(0) && pos[1] <= R(ny) &&
                       pos[2] >= R(0) && pos[2] <= R(nz))) {
@@ -595,7 +591,8 @@ __device__ __forceinline__ bool advance(const Consts &K, const HotK<R> &h, const
     if (!c.alive) return false;
     pos[0] = c.pos[0]; pos[1] = c.pos[1]; pos[2] = c.pos[2];
     ux = c.u[0]; uy = c.u[1]; uz = c.u[2];
-    ig = inverse_gamma();
+    if constexpr (kByDirection) ig = m_rsqrt(R(1) + ux * ux + uy * uy + uz * uz);
+    else ig = R(1) / m_sqrt(R(1) + ux * ux + uy * uy + uz * uz);
   }
   X = pos[0]; Y = pos[1]; Zc = pos[2];
 
